@@ -140,3 +140,16 @@ def test_accumulate_in_one_call_equals_the_per_token_calls(kind, fmt):
     assert torch.equal(E1, E2)
     assert torch.equal(G1, G2)
     assert damp.device_status() == 0
+
+
+@pytest.mark.parametrize("kda", [False, True])
+@pytest.mark.parametrize("rows", [1, 63, 64, 65, 447, 512, 577, 1500])
+def test_log_decay_sums_in_row_order(rows, kda):
+    """Every accumulator adds its rows one after the other in FP32, whatever the ring's stages."""
+    H, dk = 35 if not kda else 3, 64
+    L = damp.Layout(H, H, dk, 64, 0, 0)
+    rng = np.random.default_rng(rows)
+    g = (-np.exp(rng.uniform(-6, 0, (rows, H, dk) if kda else (rows, H)))).astype(np.float32)
+    G = damp.calib_log_decay(L, P.to_dev(g, DEV), torch.zeros((H, dk), device=DEV)).cpu().numpy()
+    ref = np.add.accumulate(g, axis=0, dtype=np.float32)[-1]
+    assert np.array_equal(G, ref if kda else np.repeat(ref[:, None], dk, axis=1))
