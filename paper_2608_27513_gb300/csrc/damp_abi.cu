@@ -1,5 +1,6 @@
 // damp_abi.cu -- the extern "C" entry points of libdamp (include/damp.h):
 // host-side argument checks, then one launch on the caller's stream.
+#include <algorithm>
 #include <atomic>
 #include <climits>
 
@@ -600,14 +601,17 @@ damp_status damp_calib_accumulate(const damp_layout *layout, float *S, int32_t n
     a.o = nullptr;  // the trajectories' outputs are not needed
     a.in_bf16 = in_dtype == DAMP_IN_BF16;
     a.kda = kda ? 1 : 0;
-    for (int64_t t = 0; t < T; ++t) {
+    // one launch per run of tokens between two samples: the states stay in registers over it
+    for (int64_t t = 0; t < T;) {
+        const int64_t n = std::min<int64_t>(every - t % every, T - t);
         a.q = static_cast<const uint8_t *>(q) + t * sq;
         a.k = static_cast<const uint8_t *>(k) + t * sq;
         a.v = static_cast<const uint8_t *>(v) + t * sv;
         a.g = reinterpret_cast<const float *>(reinterpret_cast<const uint8_t *>(g) + t * sg);
         a.beta = reinterpret_cast<const float *>(reinterpret_cast<const uint8_t *>(beta) + t * sb);
-        if (launch_fp32_step(a, s) != cudaSuccess) return DAMP_ERR_CUDA;
-        if ((t + 1) % every == 0 &&
+        if (launch_fp32_run(a, (int32_t)n, s) != cudaSuccess) return DAMP_ERR_CUDA;
+        t += n;
+        if (t % every == 0 &&
             launch_calib_error_energy(S, n_docs, (int32_t)H, (int32_t)H, nullptr, (int32_t)dk, (int32_t)dv,
                                       layout->lo_format, E_acc, s) != cudaSuccess)
             return DAMP_ERR_CUDA;

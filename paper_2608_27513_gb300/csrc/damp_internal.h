@@ -66,6 +66,9 @@ cudaError_t launch_packed_kda_f8(const StepArgs &a, cudaStream_t s);
 cudaError_t launch_quad_rowabs_gdn(const StepArgs &a, cudaStream_t s);
 cudaError_t launch_quad_rowabs_kda(const StepArgs &a, cudaStream_t s);
 cudaError_t launch_fp32_step(const StepArgs &a, cudaStream_t s);
+// n_tokens consecutive tokens of every batch row on the FP32 states, without outputs
+// (operands [n_tokens][batch][...]): the same updates as n_tokens steps, bit for bit
+cudaError_t launch_fp32_run(const StepArgs &a, int32_t n_tokens, cudaStream_t s);
 cudaError_t launch_quantize(const ConvArgs &a, cudaStream_t s);
 cudaError_t launch_dequantize(const ConvArgs &a, cudaStream_t s);
 cudaError_t launch_pack_tiers(const ConvArgs &a, cudaStream_t s);

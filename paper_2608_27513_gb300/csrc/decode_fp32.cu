@@ -1,18 +1,31 @@
-// decode_fp32.cu -- in-house FP32-state decode step (the deployment baseline of
-// Sec. 6.1: FP32 recurrent-state storage), GDN and KDA.
+// decode_fp32.cu -- the FP32-state step (the deployment baseline of Sec. 6.1: FP32
+// recurrent-state storage) and the FP32 trajectories of a calibration run, GDN and KDA.
 //
-// Same tile as the packed kernel -- (slot, head, value block c): d_k rows x 32
-// columns -- but with no quantization group the thread mapping is the simple
-// one: lane j owns column j of the tile for all d_k rows, so both column
-// reductions r = S_bar^T k and o = S^T q are thread-local and every warp-wide
-// load or store of a row is one coalesced 128-byte line.  Per-channel operands
-// (k, q, decay, beta*k) are staged once per (slot, head) in shared memory and
-// read as broadcasts.  A persistent grid: every warp walks a contiguous range of
-// tiles, keeping d_k independent loads in flight.
+// A unit is up to four value blocks of one (slot, head); a CTA of four warps walks units
+// (persistent), warp w holding a tile of d_k rows x 32 columns in registers over the
+// launch's tokens (one token for a decode step).  Lane (pc, cg) = (lane / 8, lane % 8) holds
+// columns 4 cg .. 4 cg + 3 of the rows u = pc mod 4:
+//   * a row is 128 bytes of 16-byte accesses (whole lines in memory, no bank conflicts);
+//   * the sums over the rows run as four chains (rows 0, 4, 8, ..; 1, 5, 9, ..; ...), one
+//     per lane quarter, which meet by two shuffles as (c0 + c1) + (c2 + c3);
+//   * a lane reads the operands of its own d_k / 4 rows only and uses each for four
+//     columns: 24 (KDA) 16-byte shared loads per token and tile instead of 96 with one
+//     column per lane, which were the limit of a multi-token launch.
+// The next unit's state lands in shared memory by bulk copies while the current one is
+// computed from registers and stored; the per-channel operands (k, q, decay, beta k) are
+// staged once per unit and NT tokens from copies made in the same way.
+//
+// Measured (B = 64, H = 32, d = 128, GDN, 268 MB of state per step, more than L2): 46.9 us, 5.8
+// TB/s, bound by HBM; 49.6 us with one column per lane and each tile loaded, computed and
+// stored in turn.  A calibration run over 32 documents (KDA): ~22 us for one token (the 134 MB
+// that the states move through L2), 40 us for eight, 3.1 us per further token -- FP32
+// arithmetic (1.3 us at the FMA rate) and the operand loads, with two warps per scheduler.
+// With one launch per token the eight tokens between two samples took 165 us.
 #include "damp_common.cuh"
 #include "damp_internal.h"
 
 #include <algorithm>
+#include <climits>
 
 namespace damp {
 
@@ -25,106 +38,246 @@ struct Fp32Params {
     const void *q, *k, *v;
     const float *g, *beta;
     float *o;
-    int32_t batch, H, Hqk, dk, dv, V;
-    int64_t total_tiles;
+    int32_t batch, H, Hqk, dv, V, VG;  // VG: groups of four value blocks per (slot, head)
+    int32_t n_tokens;                  // token t's operands lie t * batch rows further on
+    int64_t units;
     uint32_t *status;
 };
 
-constexpr int kFp32Warps = 8;
+constexpr int kFp32Warps = 4;
+constexpr int kFp32Ctas = 2;    // CTAs per SM: a third (168 registers a thread) spills, step 47 -> 54 us (below)
+constexpr int kFp32Tokens = 8;  // tokens staged at a time by a calibration run
 
-template <int DK, int DV, bool KDA, bool BF16>
-__global__ void __launch_bounds__(256, 1) fp32_step_kernel(const Fp32Params p) {
-    __shared__ __align__(16) float ops[kFp32Warps][4][DK];  // k, q, a, beta*k per channel
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int nw = blockDim.x >> 5;
-    float *sk = ops[warp][0];
-    float *sq = ops[warp][1];
-    float *sa = ops[warp][2];
-    float *sb = ops[warp][3];
-
-    const int64_t gw = (int64_t)blockIdx.x * nw + warp;
-    const int64_t nwt = (int64_t)gridDim.x * nw;
-    const int64_t t0 = p.total_tiles * gw / nwt;
-    const int64_t t1 = p.total_tiles * (gw + 1) / nwt;
-    bool bad_slot = false;
-
-    for (int64_t t = t0; t < t1; ++t) {
-        const int c = (int)(t % p.V);
-        const int64_t bh = t / p.V;
-        const int h = (int)(bh % p.H);
-        const int b = (int)(bh / p.H);
-        if (t == t0 || c == 0) {
-            __syncwarp();
-            const int hq = (h * p.Hqk) / p.H;
-            const int64_t qoff = ((int64_t)b * p.Hqk + hq) * DK;
-            const float beta = p.beta[(int64_t)b * p.H + h];
-            const float alpha = KDA ? 0.f : expf(p.g[(int64_t)b * p.H + h]);
-#pragma unroll
-            for (int u = lane; u < DK; u += 32) {
-                const float kv = load_in(p.k, qoff + u, BF16);
-                sk[u] = kv;
-                sq[u] = load_in(p.q, qoff + u, BF16);
-                sa[u] = KDA ? expf(p.g[((int64_t)b * p.H + h) * DK + u]) : alpha;
-                sb[u] = beta * kv;
-            }
-            __syncwarp();
-        }
-        const int64_t slot = p.slot_idx ? (int64_t)p.slot_idx[b] : (int64_t)b;
-        if (slot < 0 || slot >= p.num_slots) {
-            bad_slot = true;
-            continue;
-        }
-        float *base = p.state + ((slot * p.H + h) * DK) * (int64_t)p.dv + c * kG + lane;
-        // a compile-time row stride (DV > 0) turns every row address into an
-        // immediate offset from one base register
-        const int64_t ld = DV > 0 ? DV : p.dv;
-        float x[DK];
-#pragma unroll
-        for (int u = 0; u < DK; ++u) x[u] = __ldcs(base + u * ld);
-        const float vj = load_in(p.v, ((int64_t)b * p.H + h) * p.dv + c * kG + lane, BF16);
-
-        // S_bar = Lambda S ; r = S_bar^T k
-        float r0 = 0.f, r1 = 0.f, r2 = 0.f, r3 = 0.f;
-#pragma unroll
-        for (int u = 0; u < DK; u += 4) {
-            const float4 a4 = *reinterpret_cast<const float4 *>(sa + u);
-            const float4 k4 = *reinterpret_cast<const float4 *>(sk + u);
-            x[u] *= a4.x;
-            x[u + 1] *= a4.y;
-            x[u + 2] *= a4.z;
-            x[u + 3] *= a4.w;
-            r0 = fmaf(x[u], k4.x, r0);
-            r1 = fmaf(x[u + 1], k4.y, r1);
-            r2 = fmaf(x[u + 2], k4.z, r2);
-            r3 = fmaf(x[u + 3], k4.w, r3);
-        }
-        const float d = vj - ((r0 + r1) + (r2 + r3));
-        // S = S_bar + beta k d^T ; o = S^T q
-        float o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
-#pragma unroll
-        for (int u = 0; u < DK; u += 4) {
-            const float4 b4 = *reinterpret_cast<const float4 *>(sb + u);
-            const float4 q4 = *reinterpret_cast<const float4 *>(sq + u);
-            x[u] = fmaf(b4.x, d, x[u]);
-            x[u + 1] = fmaf(b4.y, d, x[u + 1]);
-            x[u + 2] = fmaf(b4.z, d, x[u + 2]);
-            x[u + 3] = fmaf(b4.w, d, x[u + 3]);
-            o0 = fmaf(x[u], q4.x, o0);
-            o1 = fmaf(x[u + 1], q4.y, o1);
-            o2 = fmaf(x[u + 2], q4.z, o2);
-            o3 = fmaf(x[u + 3], q4.w, o3);
-        }
-        // a fresh copy of the row pointer keeps the compiler from holding all
-        // d_k load addresses live until the stores
-#pragma unroll
-        for (int u = 0; u < DK; ++u) __stcs(base + u * ld, x[u]);
-        if (p.o) p.o[((int64_t)b * p.H + h) * p.dv + c * kG + lane] = (o0 + o1) + (o2 + o3);  // no o: calibration runs
+// RUN: a calibration run of p.n_tokens tokens without outputs; otherwise one decode step.
+// DV > 0 fixes d_v (row addresses become immediate offsets).
+template <int DK, int DV, bool KDA, bool BF16, bool RUN>
+__global__ void __launch_bounds__(32 * kFp32Warps, kFp32Ctas) fp32_tokens_kernel(const Fp32Params p) {
+    constexpr int NT = RUN ? kFp32Tokens : 1;
+    constexpr int RP = DK / 4;  // rows per lane
+    constexpr int ESZ = BF16 ? 2 : 4;
+    extern __shared__ __align__(128) uint8_t state_buf[];  // the next unit's state, row after row
+    // staged operands: channel u = 4 i + c at [c][i], so that a lane's rows are contiguous
+    __shared__ __align__(16) float sk[NT][DK], sb[NT][DK], sa[KDA ? NT : 1][DK], sq[RUN ? 1 : NT][DK];
+    __shared__ __align__(16) float sv[NT][32 * kFp32Warps];
+    __shared__ float salpha[NT];
+    // the operands as they lie in memory (cp.async)
+    __shared__ __align__(16) uint8_t rk[NT][DK * ESZ], rq[RUN ? 1 : NT][RUN ? 16 : DK * ESZ], rv[NT][kFp32Warps * 32 * ESZ];
+    __shared__ __align__(16) float rg[NT][KDA ? DK : 4], rbeta[NT];
+    __shared__ __align__(8) uint64_t bar_mem;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nthr = DV == 128 ? 128 : blockDim.x;
+    const int pc = lane >> 3, cg = lane & 7;
+    const uint32_t bar = smem_u32(&bar_mem), sbuf = smem_u32(state_buf);
+    const int64_t ld = DV > 0 ? DV : p.dv;
+    const int H = p.H, VG = p.VG;
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        fence_mbar_init();
     }
-    if (bad_slot && lane == 0) atomicOr(p.status, (uint32_t)kDevBadSlot);
+    __syncthreads();
+
+    struct Unit {
+        int64_t slot;
+        int b, h, c0, ncol;  // batch row, head, first value block, value columns
+        bool ok;             // false past the last unit
+    };
+    bool bad_slot = false;
+    int64_t at = blockIdx.x;  // the next unit to look at
+    // the next unit whose slot is in the pool
+    auto next_unit = [&]() {
+        Unit n{0, 0, 0, 0, 0, false};
+        for (; at < p.units && !n.ok; at += gridDim.x) {
+            const int64_t bh = at / VG;
+            n.c0 = (int)(at - bh * VG) * kFp32Warps;
+            n.b = (int)(bh / H);
+            n.h = (int)(bh - (int64_t)n.b * H);
+            n.ncol = DV == 128 ? 128 : min(kFp32Warps, p.V - n.c0) * kG;
+            n.slot = p.slot_idx ? (int64_t)p.slot_idx[n.b] : (int64_t)n.b;
+            n.ok = n.slot >= 0 && n.slot < p.num_slots;
+            bad_slot |= !n.ok;
+        }
+        return n;
+    };
+    auto unit_base = [&](const Unit &n) { return p.state + (n.slot * H + n.h) * DK * ld + (int64_t)n.c0 * kG; };
+    auto fetch_state = [&](const Unit &n) {  // thread 0: one copy of a whole (slot, head), or one per row
+        if (tid != 0) return;
+        fence_proxy_async_smem();  // the CTA's reads of the buffer before the copies' writes
+        mbar_arrive_expect_tx(bar, (uint32_t)(DK * n.ncol * 4));
+        const float *src = unit_base(n);
+        if (VG == 1) {
+            bulk_g2s(sbuf, src, (uint32_t)(DK * n.ncol * 4), bar);
+        } else {
+            for (int u = 0; u < DK; ++u) bulk_g2s(sbuf + (uint32_t)(u * n.ncol * 4), src + u * ld, (uint32_t)(n.ncol * 4), bar);
+        }
+    };
+    auto fetch_operands = [&](const Unit &n, int t0, int nt) {  // of the tokens t0 .. t0 + nt - 1
+        constexpr int nk = DK * ESZ / 16, nq = RUN ? 0 : nk, ng = KDA ? DK / 4 : 0;
+        const int per = nk + nq + ng + n.ncol * ESZ / 16;
+        const int hq = (n.h * p.Hqk) / H;
+        for (int i = tid; i < nt * per; i += nthr) {
+            const int s = RUN ? i / per : 0;
+            int j = i - s * per;
+            const int64_t row = (int64_t)(t0 + s) * p.batch + n.b;
+            if (j < nk) {
+                cp_async16(smem_u32(rk[s]) + 16 * j, static_cast<const uint8_t *>(p.k) + (row * p.Hqk + hq) * (DK * ESZ) + 16 * j);
+            } else if ((j -= nk) < nq) {
+                cp_async16(smem_u32(rq[s]) + 16 * j, static_cast<const uint8_t *>(p.q) + (row * p.Hqk + hq) * (DK * ESZ) + 16 * j);
+            } else if ((j -= nq) < ng) {
+                cp_async16(smem_u32(rg[s]) + 16 * j, p.g + (row * H + n.h) * DK + 4 * j);
+            } else {
+                j -= ng;
+                cp_async16(smem_u32(rv[s]) + 16 * j,
+                           static_cast<const uint8_t *>(p.v) + ((row * H + n.h) * p.dv + n.c0 * kG) * ESZ + 16 * j);
+            }
+        }
+        if (tid < nt) {
+            const int64_t row = ((int64_t)(t0 + tid) * p.batch + n.b) * H + n.h;
+            cp_async4(smem_u32(&rbeta[tid]), p.beta + row);
+            if (!KDA) cp_async4(smem_u32(&rg[tid][0]), p.g + row);
+        }
+        cp_async_commit();
+    };
+
+    const int n_tokens = RUN ? p.n_tokens : 1;
+    Unit cur = next_unit();
+    if (cur.ok) {
+        fetch_state(cur);
+        fetch_operands(cur, 0, min(NT, n_tokens));
+    }
+    uint32_t parity = 0;
+    bool timed_out = false;
+    while (cur.ok) {
+        const Unit nxt = next_unit();
+        cp_async_wait_all();
+        if (!__syncthreads_and(mbar_wait_bounded(bar, parity))) {  // the state and the first tokens' operands
+            timed_out = true;
+            break;
+        }
+        parity ^= 1u;
+        const bool live = warp * kG < cur.ncol;  // the last group of a d_v that is no multiple of 128 has idle warps
+        float2 x[RP][2];
+        if (live) {
+            const uint32_t src = sbuf + (uint32_t)((pc * cur.ncol + warp * kG + 4 * cg) * 4);
+#pragma unroll
+            for (int i = 0; i < RP; ++i) {
+                const uint4 w = lds128(src + (uint32_t)(16 * i * (DV > 0 ? DV : cur.ncol)));
+                x[i][0] = make_float2(__uint_as_float(w.x), __uint_as_float(w.y));
+                x[i][1] = make_float2(__uint_as_float(w.z), __uint_as_float(w.w));
+            }
+        }
+#pragma unroll 1
+        for (int t0 = 0; t0 < n_tokens; t0 += NT) {
+            const int nt = min(NT, n_tokens - t0);
+            if (RUN && t0 > 0) {
+                cp_async_wait_all();
+                __syncthreads();  // these tokens' operands are here, the last ones' staged form is read
+            }
+            for (int u = tid; u < DK; u += nthr) {
+                const int to = (u & 3) * RP + (u >> 2);
+#pragma unroll
+                for (int s = 0; s < NT; ++s) {
+                    if (s >= nt) break;
+                    const float kv = load_in(rk[s], u, BF16);
+                    sk[s][to] = kv;
+                    sb[s][to] = rbeta[s] * kv;
+                    if (!RUN) sq[s][to] = load_in(rq[s], u, BF16);
+                    if (KDA) sa[s][to] = expf(rg[s][u]);
+                }
+            }
+            if (!KDA && tid < nt) salpha[tid] = expf(rg[tid][0]);
+            for (int j = tid; j < cur.ncol; j += nthr) {
+                for (int s = 0; s < nt; ++s) sv[s][j] = load_in(rv[s], j, BF16);
+            }
+            __syncthreads();
+            const bool last = t0 + NT >= n_tokens;
+            if (!last) {
+                fetch_operands(cur, t0 + NT, min(NT, n_tokens - t0 - NT));
+            } else if (nxt.ok) {
+                fetch_operands(nxt, 0, min(NT, n_tokens));
+            }
+            if (t0 == 0 && nxt.ok) fetch_state(nxt);  // every warp has its tile in registers
+            if (!live) continue;
+#pragma unroll 1
+            for (int s = 0; s < nt; ++s) {
+                const float *ka = sk[s] + pc * RP, *ba = sb[s] + pc * RP, *aa = sa[KDA ? s : 0] + pc * RP;
+                const float *qa = sq[RUN ? 0 : s] + pc * RP;
+                const float alpha = KDA ? 0.f : salpha[s];
+                // S_bar = Lambda S ; r = S_bar^T k
+                float2 rp[2] = {splat2(0.f), splat2(0.f)};
+#pragma unroll
+                for (int i4 = 0; i4 < RP / 4; ++i4) {
+                    const float4 k4 = *reinterpret_cast<const float4 *>(ka + 4 * i4);
+                    const float4 a4 = KDA ? *reinterpret_cast<const float4 *>(aa + 4 * i4) : make_float4(alpha, alpha, alpha, alpha);
+                    const float kk[4] = {k4.x, k4.y, k4.z, k4.w}, av[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+#pragma unroll
+                        for (int m = 0; m < 2; ++m) {
+                            float2 &w = x[4 * i4 + e][m];
+                            w = mul2(w, splat2(av[e]));
+                            rp[m] = fma2(w, splat2(kk[e]), rp[m]);
+                        }
+                    }
+                }
+                float r[4] = {rp[0].x, rp[0].y, rp[1].x, rp[1].y};
+#pragma unroll
+                for (int m = 8; m <= 16; m <<= 1) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) r[e] += __shfl_xor_sync(kFull, r[e], m);
+                }
+                const float4 v4 = *reinterpret_cast<const float4 *>(sv[s] + warp * kG + 4 * cg);
+                const float2 d[2] = {make_float2(v4.x - r[0], v4.y - r[1]), make_float2(v4.z - r[2], v4.w - r[3])};
+                // S = S_bar + beta k d^T ; o = S^T q
+                float2 op[2] = {splat2(0.f), splat2(0.f)};
+#pragma unroll
+                for (int i4 = 0; i4 < RP / 4; ++i4) {
+                    const float4 b4 = *reinterpret_cast<const float4 *>(ba + 4 * i4);
+                    const float4 q4 = RUN ? b4 : *reinterpret_cast<const float4 *>(qa + 4 * i4);
+                    const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, qv[4] = {q4.x, q4.y, q4.z, q4.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+#pragma unroll
+                        for (int m = 0; m < 2; ++m) {
+                            float2 &w = x[4 * i4 + e][m];
+                            w = fma2(splat2(bb[e]), d[m], w);
+                            if (!RUN) op[m] = fma2(w, splat2(qv[e]), op[m]);
+                        }
+                    }
+                }
+                if (!RUN) {
+                    float o[4] = {op[0].x, op[0].y, op[1].x, op[1].y};
+#pragma unroll
+                    for (int m = 8; m <= 16; m <<= 1) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) o[e] += __shfl_xor_sync(kFull, o[e], m);
+                    }
+                    // every lane of a column group holds the sums: lane (pc, cg) writes column 4 cg + pc
+                    p.o[((int64_t)cur.b * H + cur.h) * ld + (cur.c0 + warp) * kG + 4 * cg + pc] =
+                        pc == 0 ? o[0] : pc == 1 ? o[1] : pc == 2 ? o[2] : o[3];
+                }
+            }
+        }
+        if (live) {
+            float *dst = unit_base(cur) + pc * ld + warp * kG + 4 * cg;
+#pragma unroll
+            for (int i = 0; i < RP; ++i) {
+                const float4 w = make_float4(x[i][0].x, x[i][0].y, x[i][1].x, x[i][1].y);
+                if (RUN) *reinterpret_cast<float4 *>(dst + 4 * i * ld) = w;
+                else __stcs(reinterpret_cast<float4 *>(dst + 4 * i * ld), w);
+            }
+        }
+        cur = nxt;
+    }
+    if (timed_out) mbar_wait_bounded(bar, parity);  // one more bounded wait before the buffer goes away
+    cp_async_wait_all();
+    if (tid == 0) {
+        const uint32_t bits = (timed_out ? kDevWaitTimeout : 0u) | (bad_slot ? kDevBadSlot : 0u);
+        if (bits) atomicOr(p.status, bits);
+    }
 }
 
-cudaError_t launch_fp32_step(const StepArgs &a, cudaStream_t stream) {
+template <bool RUN>
+static cudaError_t launch_fp32(const StepArgs &a, int32_t n_tokens, cudaStream_t stream) {
     Fp32Params p{};
     static std::atomic<uint32_t *> cache[64];
     cudaError_t e = symbol_address_cached(&g_status_fp32, cache, &p.status);
@@ -141,22 +294,20 @@ cudaError_t launch_fp32_step(const StepArgs &a, cudaStream_t stream) {
     p.batch = a.batch;
     p.H = a.H;
     p.Hqk = a.Hqk;
-    p.dk = a.dk;
     p.dv = a.dv;
     p.V = a.dv / kG;
-    p.total_tiles = (int64_t)a.batch * a.H * p.V;
-    if (p.total_tiles == 0) return cudaSuccess;
-    const int64_t want = (p.total_tiles + kFp32Warps - 1) / kFp32Warps;
-    const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count());
+    p.VG = (p.V + kFp32Warps - 1) / kFp32Warps;
+    p.n_tokens = n_tokens;
+    p.units = (int64_t)a.batch * a.H * p.VG;
+    if (p.units == 0 || n_tokens == 0) return cudaSuccess;
     void (*kern)(Fp32Params) = nullptr;
-#define DAMP_PICK4(DK_, DV_)                                                                   \
-    if (a.kda) kern = a.in_bf16 ? fp32_step_kernel<DK_, DV_, true, true> : fp32_step_kernel<DK_, DV_, true, false>; \
-    else kern = a.in_bf16 ? fp32_step_kernel<DK_, DV_, false, true> : fp32_step_kernel<DK_, DV_, false, false>;
-#define DAMP_PICK(DK_)                                                                         \
-    if (a.dk == DK_) {                                                                         \
-        if (a.dv == 64) { DAMP_PICK4(DK_, 64) }                                                \
-        else if (a.dv == 128) { DAMP_PICK4(DK_, 128) }                                         \
-        else { DAMP_PICK4(DK_, 0) }                                                            \
+#define DAMP_PICK4(DK_, DV_)                                                                       \
+    if (a.kda) kern = a.in_bf16 ? fp32_tokens_kernel<DK_, DV_, true, true, RUN> : fp32_tokens_kernel<DK_, DV_, true, false, RUN>; \
+    else kern = a.in_bf16 ? fp32_tokens_kernel<DK_, DV_, false, true, RUN> : fp32_tokens_kernel<DK_, DV_, false, false, RUN>;
+#define DAMP_PICK(DK_)                                                                             \
+    if (a.dk == DK_) {                                                                             \
+        if (a.dv == 128) { DAMP_PICK4(DK_, 128) }                                                  \
+        else { DAMP_PICK4(DK_, 0) }                                                                \
     }
     DAMP_PICK(32)
     DAMP_PICK(64)
@@ -164,8 +315,16 @@ cudaError_t launch_fp32_step(const StepArgs &a, cudaStream_t stream) {
 #undef DAMP_PICK
 #undef DAMP_PICK4
     if (!kern) return cudaErrorInvalidValue;
-    kern<<<grid, 32 * kFp32Warps, 0, stream>>>(p);
+    const int warps = std::min(p.V, kFp32Warps), smem = a.dk * warps * kG * 4;
+    if ((e = ensure_smem_limit(reinterpret_cast<const void *>(kern), smem)) != cudaSuccess) return e;
+    const int grid = (int)std::min<int64_t>(p.units, (int64_t)sm_count() * kFp32Ctas);
+    kern<<<grid, 32 * warps, smem, stream>>>(p);
     return cudaGetLastError();
+}
+
+cudaError_t launch_fp32_step(const StepArgs &a, cudaStream_t stream) { return launch_fp32<false>(a, 1, stream); }
+cudaError_t launch_fp32_run(const StepArgs &a, int32_t n_tokens, cudaStream_t stream) {
+    return launch_fp32<true>(a, n_tokens, stream);
 }
 
 cudaError_t take_status_fp32(uint32_t *bits) {

@@ -142,6 +142,28 @@ def test_accumulate_in_one_call_equals_the_per_token_calls(kind, fmt):
     assert damp.device_status() == 0
 
 
+@pytest.mark.parametrize("kind,dk,dv,dtype,T,every", [
+    ("kda", 128, 128, "bf16", 21, 20), ("gdn", 128, 160, "bf16", 18, 9), ("kda", 64, 32, "fp32", 8, 8),
+    ("gdn", 32, 96, "fp32", 7, 3), ("kda", 32, 256, "bf16", 3, 1), ("gdn", 64, 64, "bf16", 5, 16)])
+def test_runs_of_tokens_equal_single_steps(kind, dk, dv, dtype, T, every):
+    """The tokens between two samples run in one launch: whole and cut groups of eight staged
+    tokens, value blocks that do not fill a CTA, every d_k.  States bit for bit."""
+    w = wl.stack_layer(1 if kind == "kda" else 0, 0).replace(batch=3, heads=6, qk_heads=3, d_k=dk, d_v=dv, in_dtype=dtype)
+    L = damp.Layout(w.heads, w.qk_heads, dk, dv, 0, 0)
+    inputs = wl.torch_step_inputs(w, T, DEV)
+    st = {n: torch.stack([d[n] for d in inputs]) for n in ("q", "k", "v", "g", "beta")}
+    S1, S2 = damp.new_fp32_state(L, w.batch, DEV), damp.new_fp32_state(L, w.batch, DEV)
+    E1, E2 = (torch.zeros((w.heads, dk), device=DEV) for _ in range(2))
+    damp.calib_accumulate(L, kind, S1, st["q"], st["k"], st["v"], st["g"], st["beta"], E1, torch.zeros_like(E1), every)
+    step = damp.fp32_kda_decode_step if kind == "kda" else damp.fp32_gdn_decode_step
+    for t, d in enumerate(inputs):
+        step(L, S2, d["q"], d["k"], d["v"], d["g"], d["beta"])
+        if (t + 1) % every == 0:
+            damp.calib_error_energy(L, S2, E2)
+    assert torch.equal(S1, S2) and torch.equal(E1, E2)
+    assert damp.device_status() == 0
+
+
 @pytest.mark.parametrize("kda", [False, True])
 @pytest.mark.parametrize("rows", [1, 63, 64, 65, 447, 512, 577, 1500])
 def test_log_decay_sums_in_row_order(rows, kda):
