@@ -112,3 +112,33 @@ def test_decode_steps_small_heads(fmt, dk, dv, K):
     ragged value blocks)."""
     w = wl.Workload("t", "kda", 2, 4, 2, dk, dv, K, 1, 1, "bf16", 17, fmt)
     P.run_teacher_forced(w, 2, DEV)
+
+
+@pytest.mark.parametrize("fmt", [core.FMT_U8_H32, core.FMT_U8, *NEW])
+@pytest.mark.parametrize("dk,dv,K", [(128, 128, 128), (128, 160, 33), (64, 32, 7), (32, 96, 0)])
+def test_conversions_of_a_batch_equal_those_of_single_rows(fmt, dk, dv, K):
+    """The conversions walk 32-row items over a persistent grid: batches that no warp count
+    divides, K_hi across the item boundary, odd and at both ends, scattered slots and one slot
+    outside the pool give each row what a call of its own gives it, and FP16 rows their rounding."""
+    B, H, n = 67, 3, 70
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(dk + K)
+    S = torch.randn(B, H, dk, dv, generator=gen, device=DEV)
+    perm = torch.stack([torch.randperm(dk, generator=gen, device=DEV) for _ in range(H)]).to(torch.uint8)
+    idx = torch.randperm(n, generator=gen, device=DEV)[:B].to(torch.int32)
+    idx[11] = n
+    L = damp.Layout(H, H, dk, dv, K, fmt)
+    pool, alone = damp.new_state(L, n, DEV), damp.new_state(L, n, DEV)
+    damp.quantize_state(L, S, perm, pool, slot_idx=idx)
+    assert damp.device_status() == damp.DEV_BAD_SLOT
+    back = damp.dequantize_state(L, pool, perm, batch=B, slot_idx=idx)
+    assert damp.device_status() == damp.DEV_BAD_SLOT
+    rows = [b for b in range(B) if b != 11]
+    for b in rows:
+        damp.quantize_state(L, S[b:b + 1].contiguous(), perm, alone, slot_idx=idx[b:b + 1].clone())
+    assert torch.equal(pool, alone)
+    assert not back[11].any()
+    for b in rows[::13]:
+        assert torch.equal(back[b:b + 1], damp.dequantize_state(L, pool, perm, batch=1, slot_idx=idx[b:b + 1].clone()))
+    hi = perm[:, :K].long()[None, :, :, None].expand(len(rows), H, K, dv)
+    assert torch.equal(torch.gather(back[rows], 2, hi), torch.gather(S[rows].half().float(), 2, hi))
