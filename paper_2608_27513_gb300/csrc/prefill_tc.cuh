@@ -16,7 +16,8 @@
 // accumulation in tensor memory, M = 128):
 //     [K; Q] S_0         -> W = K S_0 (lanes 0-63), P = Q S_0 (lanes 64-127)
 //     [K; Q] K^T         -> K K^T, Q K^T
-//     [0; M] U           -> accumulated onto gamma P: O (lanes 64-127)
+//     [.; M] U           -> accumulated onto gamma P: O (lanes 64-127; rows 0-63 of the
+//                           operand are whatever their bytes hold, lanes 0-63 are not read)
 //     K^T (f_C. U)       -> accumulated onto gamma_C S_0
 // k and q are bf16 inputs (exact operands); the FP32 operands (S_0, M, U, f_C. U) enter
 // as three bf16 parts x = hi + mid + lo (24 significant bits), and a product of two split
@@ -50,7 +51,7 @@ constexpr int kSmB1 = 32768;    // S_0 as three bf16 parts, MN-major (value colu
 constexpr int kSmRec = 131072;  // the four value-block records of the (slot, head)
 constexpr int kSmV = 163840;    // v of the piece, bf16, 64 rows of 272 bytes
 constexpr int kSmA3 = 16384;    // K^T in record-row order, bf16, MN-major (16 KB)
-constexpr int kSmAO = 32768;    // [0; M] three bf16 parts, K-major (128 rows x 64 tokens, 3 x 16 KB)
+constexpr int kSmAO = 32768;    // [.; M] three bf16 parts, K-major (128 rows x 64 tokens, 3 x 16 KB)
 constexpr int kSmLP = 81920;    // L'^T (L' = L - I strictly lower), 64 rows of 68 FP32
 constexpr int kSmYU = 99328;    // Y, then U in place: 64 rows of 132 FP32
 constexpr int kSmBU = 81920;    // U as three bf16 parts, K-major (value columns x tokens, 3 x 16 KB)
@@ -133,14 +134,18 @@ __device__ __forceinline__ void split3_pair(float a, float b, uint32_t &h, uint3
     memcpy(&m, &m2, 4);
     memcpy(&l, &l2, 4);
 }
-// eight consecutive MN-elements of an operand as three 16-byte parts
-__device__ __forceinline__ void split3_store8(uint32_t dst, uint32_t part_bytes, const float *x) {
+// eight consecutive MN-elements of an operand as three 16-byte parts, off_m and off_l bytes
+// after the first (the second form: part_bytes apart)
+__device__ __forceinline__ void split3_store8(uint32_t dst, uint32_t off_m, uint32_t off_l, const float *x) {
     uint32_t h[4], m[4], l[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) split3_pair(x[2 * i], x[2 * i + 1], h[i], m[i], l[i]);
     sts128(dst, make_uint4(h[0], h[1], h[2], h[3]));
-    sts128(dst + part_bytes, make_uint4(m[0], m[1], m[2], m[3]));
-    sts128(dst + 2 * part_bytes, make_uint4(l[0], l[1], l[2], l[3]));
+    sts128(dst + off_m, make_uint4(m[0], m[1], m[2], m[3]));
+    sts128(dst + off_l, make_uint4(l[0], l[1], l[2], l[3]));
+}
+__device__ __forceinline__ void split3_store8(uint32_t dst, uint32_t part_bytes, const float *x) {
+    split3_store8(dst, part_bytes, 2 * part_bytes, x);
 }
 // byte offset of element (mn, k) in an MN-major bf16 operand whose 8-element groups
 // along MN are 128 B apart and whose 8-row groups along K are kstride apart
@@ -165,7 +170,7 @@ __device__ __forceinline__ void tc_pairs(const float (&v)[32], float2 (&y)[16]) 
 
 constexpr uint32_t kIdWP = tc_idesc(128, false, true);  // [K; Q] K-major, S_0 MN-major
 constexpr uint32_t kIdG = tc_idesc(64, false, false);   // [K; Q] and K, both K-major
-constexpr uint32_t kIdO = tc_idesc(128, false, false);  // [0; M] and U, both K-major
+constexpr uint32_t kIdO = tc_idesc(128, false, false);  // [.; M] and U, both K-major
 constexpr uint32_t kIdS = tc_idesc(128, true, false);   // K^T MN-major, f_C. U K-major
 // byte offset of element (row, k) in a K-major bf16 operand of 8-row groups 1024 B apart
 // (64 columns of K: eight 16-byte core matrices per group)
@@ -213,72 +218,84 @@ __device__ __forceinline__ void tc_reconstruct(const PrefillParams &p, uint32_t 
     }
 }
 
-// U = L^-1 Y by forward substitution for one value column, in place: col addresses row 0 of
-// the column (rows kTcRowY floats apart), lt the rows of L'^T (L' = L - I, kTcRowL floats
-// apart).  Blocks of 16 rows, 16 / NQ per part of the NQ threads that own the column: the
-// rows of a block take the solved rows of the earlier blocks (each loaded once for 16 / NQ
-// independent sums), then the parts solve their rows in turn, each first taking the rows
-// solved before it out of its own.  Every thread of the CTA calls it (NQ barriers per block).
-template <int NQ>
-__device__ __forceinline__ void tc_solve(uint32_t col, uint32_t lt, int part) {
-    constexpr int RB = 16 / NQ;  // rows per part and block (4 or 8), held as RB / 2 pairs
-    constexpr int RP = RB / 2;
-    auto ltr = [&](int srow, int t0, float2 (&lv)[RP]) {
-        const uint32_t lrow = lt + (uint32_t)(srow * kTcRowL * 4 + 4 * t0);
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// U = L^-1 Y by forward substitution, in place: yu addresses row 0 of Y (rows kTcRowY floats
+// apart), lt the rows of L'^T (L' = L - I, kTcRowL floats apart).  Warp w of NW owns the rows
+// RW w .. RW w + RW - 1 (RW = 64 / NW) of all 128 columns, lane l the columns 4 l .. 4 l + 3,
+// in registers.  Step j: warp j solves its rows among themselves and stores them; the warps
+// after it take them out of their own rows, each value of L' and of U loaded once per RW x 4
+// tile.  Every element subtracts its products in ascending row order.  Every thread of the CTA
+// calls it; the caller synchronizes after it.  Bound by the shared loads of L' and U (3840
+// cycles with 16 warps at 128 bytes a cycle): a 64-token KDA piece 8400 -> 6000 cycles against
+// a thread per column and quarter of the rows, whose every 16-byte load of L' fed four products
+// (on 8 of the 16 warps: 8000); the GDN chunk of B = 256 x 64 tokens 934 -> 878 us.
+template <int NW>
+__device__ __forceinline__ void tc_solve(uint32_t yu, uint32_t lt, int warp, int lane) {
+    constexpr int RW = kTcC / NW;  // 4 or 8
+    static_assert(RW % 4 == 0, "a warp's rows of L'^T are read in 16-byte vectors");
+    const int r0 = RW * warp;
+    const uint32_t col = yu + (uint32_t)(16 * lane), lrow = lt + (uint32_t)(4 * r0);
+    float2 acc[RW][2];
+    auto row = [&](int r, float2 (&v)[2]) {
+        const uint4 w = lds128(col + (uint32_t)(r * kTcRowY * 4));
+        v[0] = make_float2(__uint_as_float(w.x), __uint_as_float(w.y));
+        v[1] = make_float2(__uint_as_float(w.z), __uint_as_float(w.w));
+    };
+    auto ltr = [&](int s, float (&l)[RW]) {  // L' of this warp's rows at column s
 #pragma unroll
-        for (int i = 0; i < RB / 4; ++i) {
-            const uint4 l4 = lds128(lrow + 16 * i);
-            lv[2 * i] = make_float2(__uint_as_float(l4.x), __uint_as_float(l4.y));
-            lv[2 * i + 1] = make_float2(__uint_as_float(l4.z), __uint_as_float(l4.w));
+        for (int i = 0; i < RW / 4; ++i) {
+            const uint4 w = lds128(lrow + (uint32_t)(s * kTcRowL * 4 + 16 * i));
+            l[4 * i] = __uint_as_float(w.x);
+            l[4 * i + 1] = __uint_as_float(w.y);
+            l[4 * i + 2] = __uint_as_float(w.z);
+            l[4 * i + 3] = __uint_as_float(w.w);
         }
     };
-    auto row_at = [&](int r) { return col + (uint32_t)(r * kTcRowY * 4); };
+#pragma unroll
+    for (int i = 0; i < RW; ++i) row(r0 + i, acc[i]);
+    float own[RW][RW];  // L' of this warp's rows among themselves
+#pragma unroll
+    for (int a = 0; a < RW - 1; ++a) ltr(r0 + a, own[a]);
 #pragma unroll 1
-    for (int t0 = 0; t0 < kTcC; t0 += 16) {
-        const int r0 = t0 + RB * part;
-        float2 acc[RP];
+    for (int j = 0; j < warp; ++j) {
+        bar_sync(1 + (j & 1), 32 * (NW - j));  // rows RW j .. are solved
 #pragma unroll
-        for (int i = 0; i < RP; ++i) acc[i] = make_float2(ldsf(row_at(r0 + 2 * i)), ldsf(row_at(r0 + 2 * i + 1)));
-#pragma unroll 4
-        for (int s2 = 0; s2 < t0; ++s2) {
-            const float us = ldsf(row_at(s2));
-            float2 lv[RP];
-            ltr(s2, r0, lv);
+        for (int a = 0; a < RW; ++a) {
+            const int s = RW * j + a;
+            float2 u[2];
+            float l[RW];
+            row(s, u);
+            ltr(s, l);
+            u[0] = make_float2(-u[0].x, -u[0].y);
+            u[1] = make_float2(-u[1].x, -u[1].y);
 #pragma unroll
-            for (int i = 0; i < RP; ++i) acc[i] = fma2(lv[i], make_float2(-us, -us), acc[i]);
-        }
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            if (part == q) {  // own rows among themselves (the pair holding the solved row takes
-                              // zero entries of L'^T, which leave it as it is), then stored
-#pragma unroll
-                for (int a = 0; a < RB - 1; ++a) {
-                    const float ua = (a & 1) ? acc[a >> 1].y : acc[a >> 1].x;
-                    float2 lv[RP];
-                    ltr(r0 + a, r0, lv);
-#pragma unroll
-                    for (int i = a >> 1; i < RP; ++i) acc[i] = fma2(lv[i], make_float2(-ua, -ua), acc[i]);
-                }
-#pragma unroll
-                for (int i = 0; i < RP; ++i) {
-                    sts32(row_at(r0 + 2 * i), __float_as_uint(acc[i].x));
-                    sts32(row_at(r0 + 2 * i + 1), __float_as_uint(acc[i].y));
-                }
-            }
-            __syncthreads();
-            if (part > q) {  // the rows part q just solved
-#pragma unroll
-                for (int a = 0; a < RB; ++a) {
-                    const int sr = t0 + RB * q + a;
-                    const float us = ldsf(row_at(sr));
-                    float2 lv[RP];
-                    ltr(sr, r0, lv);
-#pragma unroll
-                    for (int i = 0; i < RP; ++i) acc[i] = fma2(lv[i], make_float2(-us, -us), acc[i]);
-                }
+            for (int i = 0; i < RW; ++i) {
+                acc[i][0] = fma2(splat2(l[i]), u[0], acc[i][0]);
+                acc[i][1] = fma2(splat2(l[i]), u[1], acc[i][1]);
             }
         }
     }
+#pragma unroll
+    for (int a = 0; a < RW - 1; ++a) {
+        const float2 u0 = make_float2(-acc[a][0].x, -acc[a][0].y), u1 = make_float2(-acc[a][1].x, -acc[a][1].y);
+#pragma unroll
+        for (int i = a + 1; i < RW; ++i) {
+            acc[i][0] = fma2(splat2(own[a][i]), u0, acc[i][0]);
+            acc[i][1] = fma2(splat2(own[a][i]), u1, acc[i][1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < RW; ++i)
+        sts128(col + (uint32_t)((r0 + i) * kTcRowY * 4),
+               make_uint4(__float_as_uint(acc[i][0].x), __float_as_uint(acc[i][0].y), __float_as_uint(acc[i][1].x),
+                          __float_as_uint(acc[i][1].y)));
+    if (warp < NW - 1) bar_arrive(1 + (warp & 1), 32 * (NW - warp));
 }
 
 // The chunk-final state (tensor-memory lane u = record row u, the value blocks of part
@@ -546,9 +563,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
             ph_mma ^= 1u;
             tc_fence_after();
             // ---- half 0: rows of L' = beta_t f_ts k_t.k_s (s < t; FP32, for the solve) and of
-            //      M = f_ts q_t.k_s (s <= t; rows 64 + t of [0; M], three bf16 parts), and
-            //      gamma_t P_t in tensor memory;  half 1: K^T in record-row order, the zero
-            //      rows of [0; M] and gamma_C S_0 in tensor memory ----
+            //      M = f_ts q_t.k_s (s <= t; rows 64 + t of [.; M], three bf16 parts), and
+            //      gamma_t P_t in tensor memory;  half 1: K^T in record-row order and gamma_C
+            //      S_0 in tensor memory ----
             if (half == 0) {
                 const int t = row & 63;
                 const bool qside = row >= 64;
@@ -595,10 +612,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
                     }
                 }
             } else {
-                // rows 0 .. 63 of [0; M] are zero
-#pragma unroll 1
-                for (int i = row; i < 1536; i += 128)
-                    sts128(sb + (uint32_t)(kSmAO + (i >> 9) * 16384 + (i & 511) * 16), make_uint4(0u, 0u, 0u, 0u));
                 // K^T: element (u, s) = k_s[pi(u)]; this thread takes token s = row & 63 and
                 // half the rows (its 64 channel indices first, then independent gathers)
                 {
@@ -669,8 +682,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
                 }
             }
             __syncthreads();
-            // ---- U = L^-1 Y by forward substitution (value column n = row, in place) ----
-            tc_solve<2>(sb + (uint32_t)(kSmYU + 4 * row), sb + (uint32_t)kSmLP, half);
+            // ---- U = L^-1 Y by forward substitution, in place ----
+            tc_solve<kTcThreads / 32>(sb + (uint32_t)kSmYU, sb + (uint32_t)kSmLP, warp, lane);
+            __syncthreads();
             // ---- U (half 0) and f_C. U (half 1) as three bf16 parts, K-major (value columns n x
             //      tokens s) ----
             {
@@ -693,7 +707,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
             __syncthreads();
             tc_fence_after();
             if (tid == 0) {
-                // O = gamma P + [0; M] U and S += K^T (f_C. U); six partial products of two
+                // O = gamma P + [.; M] U and S += K^T (f_C. U); six partial products of two
                 // split operands (hh, hm, mh, hl, lh, mm), three of an exact one
                 constexpr int pa[6] = {0, 0, 1, 0, 2, 1}, pb[6] = {0, 1, 0, 2, 0, 1};
 #pragma unroll

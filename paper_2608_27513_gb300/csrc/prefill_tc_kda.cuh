@@ -28,23 +28,26 @@ namespace damp {
 
 // Shared memory (bytes).  Areas that share bytes are never live together:
 //   piece inputs:   KQ [0, 34K)  XI [34K, 67K)  V [67K, 84K)   (records at unit start: [84K, 116K))
+//   piece start: EX [84K, 117K)  EN [132K, 149K)   (the exponentials of the decay ratios)
 //   per channel half: X [84K, 132K)  Z [132K, 156K)  B1 [156K, 204K)
 //   after the first products: A3 [84K, 132K)  LP [132K, 149K)  AO [149K, 197K)  YU [0, 33K)
-//   after the solve: BU [0, 48K)
+//   after the solve: BU [0, 32K) and [132K, 148K); the next piece's g and v in XI and V
 constexpr int kKdKQ = 0;            // k rows 0..63 then q rows 0..63, bf16, 272 bytes per row
 constexpr int kKdRowKQ = 272;
 constexpr int kKdXI = 34816;        // g, then xi: 64 rows of 132 FP32 (token t, channel c)
 constexpr int kKdRowXI = 132;
 constexpr int kKdV = 68608;         // v, bf16, 64 rows of 272 bytes
 constexpr int kKdRec = 86016;       // the four value-block records (unit start)
+constexpr int kKdEX = 86016;        // e^g, rows as XI
+constexpr int kKdEN = 135168;       // e^-g of the first 32 tokens, rows as XI
 constexpr int kKdX = 86016;         // X half: three bf16 parts, K-major (128 rows x 64 channels)
 constexpr int kKdZ = 135168;        // Z half: three bf16 parts, K-major (64 tokens x 64 channels)
 constexpr int kKdB1 = 159744;       // B1 half: three bf16 parts, MN-major (128 value columns x 64 channels)
 constexpr int kKdA3 = 86016;        // (K (.) Xi_C / Xi)^T: three bf16 parts, K-major (128 record rows x 64 tokens)
 constexpr int kKdLP = 135168;       // L'^T, 64 rows of kTcRowL FP32
-constexpr int kKdAO = 152576;       // [0; M]: three bf16 parts, K-major (128 rows x 64 tokens)
+constexpr int kKdAO = 152576;       // [.; M]: three bf16 parts, K-major (128 rows x 64 tokens)
 constexpr int kKdYU = 0;            // Y, then U: 64 rows of kTcRowY FP32
-constexpr int kKdBU = 0;            // U: three bf16 parts, K-major (value columns x tokens)
+__host__ __device__ constexpr int kd_bu(int part) { return part == 2 ? 135168 : 16384 * part; }  // U: three bf16 parts, K-major (value columns x tokens)
 constexpr int kKdScal = 208896;     // beta, pi, gamma_m, xi_C, mbarriers, TMEM address
 constexpr int kKdSmem = kKdScal + 2048;
 constexpr int kKdMaxRec = 8192;     // four records fit in [kKdRec, kKdZ)
@@ -114,20 +117,10 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         return n;
     };
     auto rec_of = [&](const Unit &n) { return p.state + n.slot * p.slot_bytes + (int64_t)(n.h * 4) * rec_bytes; };
-    // k, q, g, v and beta of unit n's tokens p0 .. p0 + 63 (cp.async; rows past the row's
-    // length are zero)
-    auto load_piece = [&](const Unit &n, int p0) {
+    // g, v and beta of unit n's tokens p0 .. p0 + 63 (cp.async; rows past the row's length are
+    // zero), issued while the products of the piece before run
+    auto load_gv = [&](const Unit &n, int p0) {
         const int nl = min(kTcC, n.Tb - p0);
-#pragma unroll 1
-        for (int i = tid; i < 2048; i += kKdThreads) {  // k rows 0..63, q rows 64..127: 16 chunks each
-            const int m = i >> 4, j = i & 15, t = m & 63;
-            const uint32_t dst = kq + (uint32_t)(m * kKdRowKQ + 16 * j);
-            if (t < nl)
-                cp_async16(dst, static_cast<const uint8_t *>(m < 64 ? p.k : p.q) +
-                                    (((int64_t)n.b * T + p0 + t) * p.Hqk + n.hq) * 256 + 16 * j);
-            else
-                sts128(dst, make_uint4(0u, 0u, 0u, 0u));
-        }
 #pragma unroll 1
         for (int i = tid; i < 2048; i += kKdThreads) {  // g: 64 rows of 32 chunks
             const int t = i >> 5, j = i & 31;
@@ -153,8 +146,23 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         }
         cp_async_commit();
     };
-    // unit n's records, pi and first piece, one unit ahead
-    auto prefetch = [&](const Unit &n) {
+    // its k and q (needed after the decay ratios), once the products that read U are done
+    auto load_kq = [&](const Unit &n, int p0) {
+        const int nl = min(kTcC, n.Tb - p0);
+#pragma unroll 1
+        for (int i = tid; i < 2048; i += kKdThreads) {  // k rows 0..63, q rows 64..127: 16 chunks each
+            const int m = i >> 4, j = i & 15, t = m & 63;
+            const uint32_t dst = kq + (uint32_t)(m * kKdRowKQ + 16 * j);
+            if (t < nl)
+                cp_async16(dst, static_cast<const uint8_t *>(m < 64 ? p.k : p.q) +
+                                    (((int64_t)n.b * T + p0 + t) * p.Hqk + n.hq) * 256 + 16 * j);
+            else
+                sts128(dst, make_uint4(0u, 0u, 0u, 0u));
+        }
+        cp_async_commit();
+    };
+    // unit n's records and pi, one unit ahead (their copies join load_kq's group)
+    auto load_records = [&](const Unit &n) {
         if (tid == 0) {
             fence_proxy_async_smem();
             mbar_arrive_expect_tx(bar_rec, (uint32_t)(4 * rec_bytes));
@@ -164,12 +172,15 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
                 bulk_g2s(sb + (uint32_t)(kKdRec + c * rstride), g0 + (int64_t)c * rec_bytes, (uint32_t)rec_bytes, bar_rec);
         }
         if (tid < 8) cp_async16(s_perm + 16 * tid, p.perm + (int64_t)n.h * 128 + 16 * tid);
-        load_piece(n, 0);
         rec_pending = true;
     };
 
     Unit cur = next_unit(blockIdx.x);
-    if (cur.unit < units) prefetch(cur);
+    if (cur.unit < units) {
+        load_gv(cur, 0);
+        load_records(cur);
+        load_kq(cur, 0);
+    }
     while (cur.unit < units) {
         const int b = cur.b, Tb = cur.Tb, mh = cur.mh;
         uint8_t *const grec0 = rec_of(cur);
@@ -185,12 +196,9 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         __syncthreads();  // the records are read: the first piece's operands go over them
 
         int p0 = 0;
-        bool first = true;
 #pragma unroll 1
         while (p0 < Tb) {
-            if (!first) load_piece(cur, p0);
-            first = false;
-            cp_async_wait_all();
+            cp_async_wait<1>();  // g, v and beta (k and q may still be on their way)
             __syncthreads();
             // ---- the piece's length: the largest of 64, 32, ..., 1 tokens over which every
             //      channel decays by at most e^kKdMaxLog on either side of the reference
@@ -209,6 +217,17 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
                     if (t == 31) lam[5] = acc;
                     if (t == 63) lam[6] = acc;
                 }
+            } else {
+                // meanwhile the other quarters take the exponentials (a reference token is at
+                // most token 31): the running products below are then one product per token
+                const uint32_t col = (uint32_t)(4 * row);
+#pragma unroll 4
+                for (int j = qq - 1; j < 96; j += 3) {
+                    const int t = j < 64 ? j : j - 64;
+                    const float g = ldsf(xi + (uint32_t)(t * kKdRowXI * 4) + col);
+                    const float e = expf(j < 64 ? g : -g);
+                    sts32(sb + (uint32_t)((j < 64 ? kKdEX : kKdEN) + t * kKdRowXI * 4) + col, __float_as_uint(e));
+                }
             }
             int L = 1;
 #pragma unroll
@@ -219,34 +238,36 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
             const int nt = min(L, Tb - p0);   // tokens of this piece; the rest are masked
             const int m = L > 1 ? L / 2 - 1 : 0;
             // ---- xi_t = gamma_t / gamma_m in place of g (0 for masked tokens), as running
-            //      products from m (quarter 0: downward, xi_{t-1} = xi_t e^{-g_t}, and gamma_m;
-            //      quarter 1: upward, xi_t = xi_{t-1} e^{g_t}); xi_C at C = nt - 1 ----
+            //      products from m (quarter 0: downward, xi_{t-1} = xi_t e^{-g_t}; quarter 1:
+            //      upward, xi_t = xi_{t-1} e^{g_t}; quarter 2: gamma_m); xi_C at C = nt - 1
+            //      (the first barrier of the length's choice has published the exponentials) ----
             {
-                const uint32_t colc = xi + (uint32_t)(4 * row);
+                const uint32_t col = (uint32_t)(4 * row), colc = xi + col;
+                const uint32_t ex = sb + (uint32_t)kKdEX + col, en = sb + (uint32_t)kKdEN + col;
+                constexpr uint32_t kR = kKdRowXI * 4;
                 float x = 1.f;
                 if (qq == 0) {
-                    float gm = 1.f;
-#pragma unroll 1
+#pragma unroll 4
                     for (int t = m; t >= 0; --t) {
-                        const uint32_t a = colc + (uint32_t)(t * kKdRowXI * 4);
-                        const float g = ldsf(a);
-                        sts32(a, __float_as_uint(t < nt ? x : 0.f));
-                        if (t == nt - 1) sts32(s_xiC + 4 * row, __float_as_uint(x));
-                        gm *= expf(g);
-                        x *= expf(-g);
+                        sts32(colc + t * kR, __float_as_uint(t < nt ? x : 0.f));
+                        if (t == nt - 1) sts32(s_xiC + col, __float_as_uint(x));
+                        x *= ldsf(en + t * kR);
                     }
-                    sts32(s_gm + 4 * row, __float_as_uint(gm));
                 } else if (qq == 1) {
-#pragma unroll 1
+#pragma unroll 4
                     for (int t = m + 1; t < kTcC; ++t) {
-                        const uint32_t a = colc + (uint32_t)(t * kKdRowXI * 4);
-                        x *= expf(ldsf(a));
-                        sts32(a, __float_as_uint(t < nt ? x : 0.f));
-                        if (t == nt - 1) sts32(s_xiC + 4 * row, __float_as_uint(x));
+                        x *= ldsf(ex + t * kR);
+                        sts32(colc + t * kR, __float_as_uint(t < nt ? x : 0.f));
+                        if (t == nt - 1) sts32(s_xiC + col, __float_as_uint(x));
                     }
+                } else if (qq == 2) {
+#pragma unroll 4
+                    for (int t = m; t >= 0; --t) x *= ldsf(ex + t * kR);
+                    sts32(s_gm + col, __float_as_uint(x));
                 }
             }
             if (tid < kTcC && tid >= nt) sts32(s_beta + 4 * tid, 0u);  // tokens past the piece
+            cp_async_wait_all();  // k and q
             __syncthreads();
             // ---- per channel half (64 channels): X = [K (.) Xi; Q (.) Xi], Z = K / Xi and
             //      B1 = diag(gamma_m) S_0 as three bf16 parts; W | P += X B1 and the Gram rows
@@ -336,51 +357,46 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
                 tc_fence_after();
             }
             if (timed_out) break;
-            // ---- quarter 0: rows of L' = beta_t G_ts (s < t) and M = G_ts (s <= t) from the
-            //      Gram rows (the decay is in G); quarter 1: the zero rows of [0; M]; all:
-            //      (K (.) Xi_C / Xi)^T in record-row order and gamma_C S_0 in tensor memory ----
-            if (qq == 0) {
+            // ---- quarters 0 and 1: rows of L' = beta_t G_ts (s < t) and M = G_ts (s <= t) from the
+            //      Gram rows (the decay is in G), columns s of 32 qq .. 32 qq + 31; all: the
+            //      state-update operand and gamma_C S_0 in tensor memory ----
+            if (qq < 2) {
                 const int t = row & 63;
                 const bool qside = row >= 64;
                 const float bt = qside ? 1.f : ldsf(s_beta + 4 * t);
-#pragma unroll 1
-                for (int h2 = 0; h2 < 2; ++h2) {  // columns s of 32 h2 .. 32 h2 + 31
-                    float gr[32];
-                    tc_ld32(tG + 32 * h2, gr);
+                float gr[32];
+                tc_ld32(tG + 32 * qq, gr);
 #pragma unroll
-                    for (int s2 = 0; s2 < 32; ++s2) {
-                        const int sc = 32 * h2 + s2;
-                        gr[s2] = sc < t ? bt * gr[s2] : (sc == t && qside ? gr[s2] : 0.f);
-                    }
-                    if (!qside) {  // column t of L'^T
-                        const uint32_t colt = sb + (uint32_t)(kKdLP + 4 * t + 32 * h2 * kTcRowL * 4);
-#pragma unroll
-                        for (int s2 = 0; s2 < 32; ++s2) sts32(colt + (uint32_t)(s2 * kTcRowL * 4), __float_as_uint(gr[s2]));
-                    } else {
-#pragma unroll
-                        for (int g = 0; g < 4; ++g)
-                            split3_store8(sb + kKdAO + tc_k64_off(64 + t, 32 * h2 + 8 * g), 16384, gr + 8 * g);
-                    }
+                for (int s2 = 0; s2 < 32; ++s2) {
+                    const int sc = 32 * qq + s2;
+                    gr[s2] = sc < t ? bt * gr[s2] : (sc == t && qside ? gr[s2] : 0.f);
                 }
-            } else if (qq == 1) {
-#pragma unroll 1
-                for (int i = row; i < 1536; i += 128)
-                    sts128(sb + (uint32_t)(kKdAO + (i >> 9) * 16384 + (i & 511) * 16), make_uint4(0u, 0u, 0u, 0u));
+                if (!qside) {  // column t of L'^T
+                    const uint32_t colt = sb + (uint32_t)(kKdLP + 4 * t + 32 * qq * kTcRowL * 4);
+#pragma unroll
+                    for (int s2 = 0; s2 < 32; ++s2) sts32(colt + (uint32_t)(s2 * kTcRowL * 4), __float_as_uint(gr[s2]));
+                } else {
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        split3_store8(sb + kKdAO + tc_k64_off(64 + t, 32 * qq + 8 * g), 16384, gr + 8 * g);
+                }
             }
-            {  // (K (.) Xi_C / Xi)^T, K-major: record row u = row (channel pi(u)), tokens 16 qq .. + 15
+            {  // (K (.) Xi_C / Xi)^T, K-major: record row u = row (channel pi(u)); 8 tokens in quarters
+               // 0 and 1, 24 in quarters 2 and 3
                 const uint32_t ch = lds_u8(s_perm + row) & 127u;
                 const float xic = ldsf(s_xiC + 4u * ch);
-#pragma unroll
-                for (int g8 = 0; g8 < 2; ++g8) {
+                const int ta = qq < 2 ? 8 * qq : 24 * qq - 32, tb = ta + (qq < 2 ? 8 : 24);
+#pragma unroll 1
+                for (int t8 = ta; t8 < tb; t8 += 8) {
                     float v[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const int t = 16 * qq + 8 * g8 + e;
+                        const int t = t8 + e;
                         const float kv = __uint_as_float(lds_u16(kq + (uint32_t)(t * kKdRowKQ) + 2u * ch) << 16);
                         const float xs = ldsf(xi + (uint32_t)(t * kKdRowXI * 4) + 4u * ch);
                         v[e] = xs != 0.f ? kv * (xic * __frcp_rn(xs)) : 0.f;  // masked tokens: 0
                     }
-                    split3_store8(sb + kKdA3 + tc_k64_off(row, 16 * qq + 8 * g8), 16384, v);
+                    split3_store8(sb + kKdA3 + tc_k64_off(row, t8), 16384, v);
                 }
             }
             {  // gamma_C S_0 = gamma_m xi_C S_0 (per channel; the state product accumulates onto it)
@@ -425,8 +441,13 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
                 }
             }
             __syncthreads();
-            // ---- U = L^-1 Y (value column n = row, in place) ----
-            tc_solve<4>(sb + (uint32_t)(kKdYU + 4 * row), sb + (uint32_t)kKdLP, qq);
+            // g, v and beta are read: the next piece's go over them
+            const bool last = p0 + nt >= Tb;
+            if (!last) load_gv(cur, p0 + nt);
+            else if (nxt.unit < units) load_gv(nxt, 0);
+            // ---- U = L^-1 Y, in place ----
+            tc_solve<kKdThreads / 32>(sb + (uint32_t)kKdYU, sb + (uint32_t)kKdLP, warp, lane);
+            __syncthreads();
             // ---- U as three bf16 parts, K-major (value columns n x tokens s): tokens 16 qq .. + 15 ----
             {
                 const uint32_t col = sb + (uint32_t)(kKdYU + 4 * row);
@@ -435,27 +456,27 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
                 for (int t = 0; t < 16; ++t) uc[t] = ldsf(col + (uint32_t)((16 * qq + t) * kTcRowY * 4));
                 __syncthreads();  // every column is read: the parts go over Y / U
 #pragma unroll
-                for (int g = 0; g < 2; ++g) split3_store8(sb + kKdBU + tc_k64_off(row, 16 * qq + 8 * g), 16384, uc + 8 * g);
+                for (int g = 0; g < 2; ++g) split3_store8(sb + tc_k64_off(row, 16 * qq + 8 * g), kd_bu(1), kd_bu(2), uc + 8 * g);
             }
             fence_proxy_async_smem();
             tc_fence_before();
             __syncthreads();
             tc_fence_after();
             if (tid == 0) {
-                // O = P + [0; M] U and S += (K (.) Xi_C / Xi)^T U; six partial products each
+                // O = P + [.; M] U and S += (K (.) Xi_C / Xi)^T U; six partial products each
                 constexpr int pa[6] = {0, 0, 1, 0, 2, 1}, pb[6] = {0, 1, 0, 2, 0, 1};
 #pragma unroll
                 for (int q = 0; q < 6; ++q)
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
                         tc_mma(tmem + kColWP, tc_desc(sb + kKdAO + 16384 * pa[q] + 256 * ks, 128, 1024),
-                               tc_desc(sb + kKdBU + 16384 * pb[q] + 256 * ks, 128, 1024), kIdO, 1u);
+                               tc_desc(sb + kd_bu(pb[q]) + 256 * ks, 128, 1024), kIdO, 1u);
 #pragma unroll
                 for (int q = 0; q < 6; ++q)
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
                         tc_mma(tmem + kColS, tc_desc(sb + kKdA3 + 16384 * pa[q] + 256 * ks, 128, 1024),
-                               tc_desc(sb + kKdBU + 16384 * pb[q] + 256 * ks, 128, 1024), kIdO, 1u);
+                               tc_desc(sb + kd_bu(pb[q]) + 256 * ks, 128, 1024), kIdO, 1u);
                 tc_commit(bar_mma);
             }
             if (!tc_wait_all(bar_mma, ph_mma)) {
@@ -464,7 +485,13 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
             }
             ph_mma ^= 1u;
             tc_fence_after();
-            if (p0 + nt >= Tb && nxt.unit < units) prefetch(nxt);  // the next unit's loads overlap this one's tail
+            // the next piece's or unit's loads overlap this one's tail
+            if (!last) {
+                load_kq(cur, p0 + nt);
+            } else if (nxt.unit < units) {
+                load_records(nxt);
+                load_kq(nxt, 0);
+            }
             // ---- o_t = H (P_t + (M U)_t) (lanes 64 + t, this quarter's value block) ----
             if (row >= 64) {
                 const int t = row - 64;
