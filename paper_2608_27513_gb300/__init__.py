@@ -18,6 +18,7 @@ pool and permutation table per K_hi, each with a head map into the layer's heads
 from __future__ import annotations
 
 import ctypes
+import functools
 from dataclasses import dataclass, field
 
 from ._lib import DampLayout, DampLibraryError, lib
@@ -86,6 +87,26 @@ class Layout:
                           self.model_heads, None if self.head_map is None else self.head_map.data_ptr())
 
 
+# The struct of a layout and its slot size depend on the layout's values alone (the head map
+# enters with the address it has at the call), and the library only reads the struct: both are
+# kept by value.
+@functools.lru_cache(maxsize=512)
+def _layout_of(H, Hqk, dk, dv, k_hi, fmt, Hm, head_map):
+    return ctypes.pointer(DampLayout(H, Hqk, dk, dv, k_hi, fmt, Hm, head_map))
+
+
+def _cptr(layout):
+    m = layout.head_map
+    return _layout_of(layout.num_heads, layout.num_qk_heads, layout.d_k, layout.d_v, layout.k_hi, layout.lo_format,
+                      layout.model_heads, None if m is None else m.data_ptr())
+
+
+@functools.lru_cache(maxsize=512)
+def _slot_bytes_of(H, Hqk, dk, dv, k_hi, fmt, Hm, mapped):
+    """Slot size of a pool, 0 for a layout the library does not take (a map's address plays no part)."""
+    return int(lib().damp_slot_bytes(ctypes.pointer(DampLayout(H, Hqk, dk, dv, k_hi, fmt, Hm, 16 if mapped else None))))
+
+
 def head_groups(k_hi_of_head, num_qk_heads: int, d_k: int, d_v: int, lo_format: int = LO_U8_AFFINE_G32_H32,
                 device="cuda"):
     """Layouts of a layer whose heads keep different numbers of FP16 key channels
@@ -113,6 +134,51 @@ def _stream(stream):
     return ctypes.c_void_p(s.cuda_stream)
 
 
+def _raw_stream(torch, stream):
+    """The cudaStream_t of a call as an integer: the given stream's, or the current one's."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+# Every call checks all its tensors (shape, dtype, device, contiguity).  _fits* take the usual
+# case in a few comparisons; a tensor that does not fit is left to the checks below, which
+# name it.  (A decode step of one request spent 30 us on the host with those checks alone, 11 us
+# of device time included.)
+def _fit(t, shape, dtype):
+    return t.shape == shape and t.dtype is dtype and t.is_cuda and t.is_contiguous()
+
+
+def _fits_operands(torch, layout, kda, q, k, v, g, beta, o, slot_idx, lead):
+    Hm, dt, f32 = layout.model_heads or layout.num_heads, v.dtype, torch.float32
+    qk = lead + (layout.num_qk_heads, layout.d_k)
+    vo, gh = lead + (Hm, layout.d_v), lead + (Hm,)
+    return ((dt is torch.bfloat16 or dt is f32) and _fit(q, qk, dt) and _fit(k, qk, dt) and _fit(v, vo, dt)
+            and _fit(g, gh + (layout.d_k,) if kda else gh, f32) and _fit(beta, gh, f32)
+            and (o is None or _fit(o, vo, f32)) and (slot_idx is None or _fit(slot_idx, lead[:1], torch.int32)))
+
+
+def _fits_pool(torch, layout, state, perm, num_slots, B, slot_idx):
+    """state and perm of a packed call, and num_slots (None: all of state's)."""
+    n = state.shape[0]
+    sb = _slot_bytes_of(layout.num_heads, layout.num_qk_heads, layout.d_k, layout.d_v, layout.k_hi, layout.lo_format,
+                        layout.model_heads, layout.head_map is not None)
+    return (sb > 0 and (num_slots is None or 0 <= num_slots <= n)
+            and (slot_idx is not None or B <= (n if num_slots is None else num_slots))
+            and _fit(state, (n, sb), torch.uint8) and _fit(perm, (layout.num_heads, layout.d_k), torch.uint8))
+
+
+def _fits_fp32(torch, layout, state, num_slots, B, slot_idx):
+    n = state.shape[0]
+    return ((num_slots is None or 0 <= num_slots <= n)
+            and (slot_idx is not None or B <= (n if num_slots is None else num_slots))
+            and _fit(state, (n, layout.num_heads, layout.d_k, layout.d_v), torch.float32))
+
+
+def _addr(t):
+    return None if t is None else t.data_ptr()
+
+
 def _check(status: int, what: str):
     if status != 0:
         raise DampError(status, what)
@@ -120,6 +186,9 @@ def _check(status: int, what: str):
 
 def _in_dtype(*ts) -> int:
     import torch
+    d0 = ts[0].dtype
+    if d0 is torch.bfloat16 and all(t.dtype is d0 for t in ts):
+        return IN_BF16
     dts = {t.dtype for t in ts}
     if dts == {torch.bfloat16}:
         return IN_BF16
@@ -227,27 +296,36 @@ def new_fp32_state(layout: Layout, num_slots: int, device="cuda"):
 def _step(fn_name, layout, state, perm, q, k, v, g, beta, o, slot_idx, num_slots, stream):
     import torch
     fp32 = fn_name.startswith("damp_fp32")
+    kda = "_kda_" in fn_name
     if v is None or v.dim() < 1:
         raise ValueError("v must be a [B, H, d_v] tensor")
     B = v.shape[0]
-    num_slots = _want_pool(layout, state, num_slots, fp32=fp32)
-    _want_batch(slot_idx, B, num_slots)
-    if not fp32:
-        _want("perm", perm, (layout.num_heads, layout.d_k), dtype=torch.uint8)
-    _want_operands(layout, "kda" if "_kda_" in fn_name else "gdn", q, k, v, g, beta, o, (B,))
-    for n, t in (("state", state), ("perm", perm), ("q", q), ("k", k), ("v", v), ("g", g), ("beta", beta),
-                 ("o", o), ("slot_idx", slot_idx)):
-        _cuda_contig(n, t)
+    try:
+        fits = (_fits_fp32(torch, layout, state, num_slots, B, slot_idx) if fp32 else
+                _fits_pool(torch, layout, state, perm, num_slots, B, slot_idx)) and _fits_operands(
+            torch, layout, kda, q, k, v, g, beta, o, slot_idx, (B,))
+    except (AttributeError, IndexError, TypeError):  # a missing tensor, or one of another kind
+        fits = False
+    if fits:
+        num_slots = state.shape[0] if num_slots is None else int(num_slots)
+    else:
+        num_slots = _want_pool(layout, state, num_slots, fp32=fp32)
+        _want_batch(slot_idx, B, num_slots)
+        if not fp32:
+            _want("perm", perm, (layout.num_heads, layout.d_k), dtype=torch.uint8)
+        _want_operands(layout, "kda" if kda else "gdn", q, k, v, g, beta, o, (B,))
+        for n, t in (("state", state), ("perm", perm), ("q", q), ("k", k), ("v", v), ("g", g), ("beta", beta),
+                     ("o", o), ("slot_idx", slot_idx)):
+            _cuda_contig(n, t)
     if o is None:
         # a head group writes only its heads' rows: the others start at zero
-        alloc = torch.empty if layout.head_map is None else torch.zeros
-        o = alloc((B, layout.heads_of_operands, layout.d_v), dtype=torch.float32, device=v.device)
-    c = layout.c()
-    args = [ctypes.byref(c), _ptr(state), num_slots, _ptr(slot_idx), B]
-    if perm is not None or not fn_name.startswith("damp_fp32"):
-        args.append(_ptr(perm))
-    args += [_ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(o), _in_dtype(q, k, v), _stream(stream)]
-    _check(getattr(lib(), fn_name)(*args), fn_name)
+        alloc = v.new_empty if layout.head_map is None else v.new_zeros
+        o = alloc((B, layout.heads_of_operands, layout.d_v), dtype=torch.float32)
+    tail = (q.data_ptr(), k.data_ptr(), v.data_ptr(), g.data_ptr(), beta.data_ptr(), o.data_ptr(), _in_dtype(q, k, v),
+            _raw_stream(torch, stream))
+    head = (_cptr(layout), state.data_ptr(), num_slots, _addr(slot_idx), B)
+    fn = getattr(lib(), fn_name)
+    _check(fn(*head, *tail) if fp32 else fn(*head, _addr(perm), *tail), fn_name)
     return o
 
 
@@ -275,25 +353,35 @@ def _step_groups(fn_name, groups, q, k, v, g, beta, o, slot_idx, stream):
     states = (ctypes.c_void_p * n)()
     perms = (ctypes.c_void_p * n)()
     slots = (ctypes.c_int64 * n)()
+    kda = kind == "kda"
+    try:
+        fits = all(layout.head_map is not None and _fits_pool(torch, layout, state, perm, None, B, slot_idx)
+                   and _fits_operands(torch, layout, kda, q, k, v, g, beta, o, slot_idx, (B,))
+                   for layout, state, perm in groups)
+    except (AttributeError, IndexError, TypeError):  # a missing tensor, or one of another kind
+        fits = False
     for i, (layout, state, perm) in enumerate(groups):
-        if layout.head_map is None:
-            raise ValueError(f"group {i} has no head map (build the groups with head_groups)")
-        ns = _want_pool(layout, state, None)
-        _want_batch(slot_idx, B, ns)
-        _want("perm", perm, (layout.num_heads, layout.d_k), dtype=torch.uint8)
-        _want_operands(layout, kind, q, k, v, g, beta, o, (B,))
-        _cuda_contig("state", state)
-        _cuda_contig("perm", perm)
+        if not fits:
+            if layout.head_map is None:
+                raise ValueError(f"group {i} has no head map (build the groups with head_groups)")
+            ns = _want_pool(layout, state, None)
+            _want_batch(slot_idx, B, ns)
+            _want("perm", perm, (layout.num_heads, layout.d_k), dtype=torch.uint8)
+            _want_operands(layout, kind, q, k, v, g, beta, o, (B,))
+            _cuda_contig("state", state)
+            _cuda_contig("perm", perm)
         layouts[i] = layout.c()
         states[i] = state.data_ptr()
         perms[i] = perm.data_ptr()
-        slots[i] = ns
-    for nm, t in (("q", q), ("k", k), ("v", v), ("g", g), ("beta", beta), ("o", o), ("slot_idx", slot_idx)):
-        _cuda_contig(nm, t)
+        slots[i] = state.shape[0]
+    if not fits:
+        for nm, t in (("q", q), ("k", k), ("v", v), ("g", g), ("beta", beta), ("o", o), ("slot_idx", slot_idx)):
+            _cuda_contig(nm, t)
     if o is None:
-        o = torch.empty((B, groups[0][0].heads_of_operands, groups[0][0].d_v), dtype=torch.float32, device=v.device)
-    _check(getattr(lib(), fn_name)(layouts, n, states, slots, perms, _ptr(slot_idx), B, _ptr(q), _ptr(k), _ptr(v),
-                                   _ptr(g), _ptr(beta), _ptr(o), _in_dtype(q, k, v), _stream(stream)), fn_name)
+        o = v.new_empty((B, groups[0][0].heads_of_operands, groups[0][0].d_v), dtype=torch.float32)
+    _check(getattr(lib(), fn_name)(layouts, n, states, slots, perms, _addr(slot_idx), B, q.data_ptr(), k.data_ptr(),
+                                   v.data_ptr(), g.data_ptr(), beta.data_ptr(), o.data_ptr(), _in_dtype(q, k, v),
+                                   _raw_stream(torch, stream)), fn_name)
     return o
 
 
@@ -339,20 +427,33 @@ def _prefill(fn_name, layout, state, perm, q, k, v, g, beta, o, lengths, slot_id
     if v is None or v.dim() < 2:
         raise ValueError("v must be a [B, T, H, d_v] tensor")
     B, T = v.shape[0], v.shape[1]
-    num_slots = _want_pool(layout, state, num_slots)
-    _want_batch(slot_idx, B, num_slots)
-    _want("lengths", lengths, (B,), dtype=torch.int32)
-    _want("perm", perm, (layout.num_heads, layout.d_k), dtype=torch.uint8)
-    _want_operands(layout, "kda" if "_kda_" in fn_name else "gdn", q, k, v, g, beta, o, (B, T))
-    for n, t in (("state", state), ("perm", perm), ("q", q), ("k", k), ("v", v), ("g", g), ("beta", beta),
-                 ("o", o), ("lengths", lengths), ("slot_idx", slot_idx)):
-        _cuda_contig(n, t)
+    kda = "_kda_" in fn_name
+    try:
+        fits = _fits_pool(torch, layout, state, perm, num_slots, B, slot_idx) and _fits_operands(
+            torch, layout, kda, q, k, v, g, beta, o, slot_idx, (B, T)) and (
+            lengths is None or _fit(lengths, (B,), torch.int32))
+    except (AttributeError, IndexError, TypeError):  # a missing tensor, or one of another kind
+        fits = False
+    if fits:
+        num_slots = state.shape[0] if num_slots is None else int(num_slots)
+    else:
+        num_slots = _want_pool(layout, state, num_slots)
+        _want_batch(slot_idx, B, num_slots)
+        _want("lengths", lengths, (B,), dtype=torch.int32)
+        _want("perm", perm, (layout.num_heads, layout.d_k), dtype=torch.uint8)
+        _want_operands(layout, "kda" if kda else "gdn", q, k, v, g, beta, o, (B, T))
+        for n, t in (("state", state), ("perm", perm), ("q", q), ("k", k), ("v", v), ("g", g), ("beta", beta),
+                     ("o", o), ("slot_idx", slot_idx), ("lengths", lengths)):
+            _cuda_contig(n, t)
     if o is None:
-        o = torch.zeros((B, T, layout.heads_of_operands, layout.d_v), dtype=torch.float32, device=v.device)
-    c = layout.c()
-    _check(getattr(lib(), fn_name)(ctypes.byref(c), _ptr(state), num_slots, _ptr(slot_idx), B, T, _ptr(lengths),
-                                   _ptr(perm), _ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(o),
-                                   _in_dtype(q, k, v), _stream(stream)), fn_name)
+        # rows past a length, of a slot outside the pool or of another group's heads stay zero;
+        # without lengths, slot indices and a head map the call writes every row
+        alloc = v.new_empty if lengths is None and slot_idx is None and layout.head_map is None else v.new_zeros
+        o = alloc((B, T, layout.heads_of_operands, layout.d_v), dtype=torch.float32)
+    _check(getattr(lib(), fn_name)(_cptr(layout), state.data_ptr(), num_slots, _addr(slot_idx), B, T, _addr(lengths),
+                                   _addr(perm), q.data_ptr(), k.data_ptr(), v.data_ptr(), g.data_ptr(),
+                                   beta.data_ptr(), o.data_ptr(), _in_dtype(q, k, v), _raw_stream(torch, stream)),
+           fn_name)
     return o
 
 
@@ -446,15 +547,24 @@ def quantize_state(layout, S, perm, state, slot_idx=None, num_slots=None, stream
     import torch
     if S is None or S.dim() != 4:
         raise ValueError("S must be a [B, H, d_k, d_v] tensor")
-    n_slots = _want_pool(layout, state, num_slots)
-    _want_batch(slot_idx, S.shape[0], n_slots)
-    _want("S", S, (S.shape[0], layout.heads_of_operands, layout.d_k, layout.d_v), dtype=torch.float32)
-    _want("perm", perm, (layout.num_heads, layout.d_k), dtype=torch.uint8)
-    for n, t in (("S", S), ("perm", perm), ("state", state), ("slot_idx", slot_idx)):
-        _cuda_contig(n, t)
-    c = layout.c()
-    _check(lib().damp_quantize_state(ctypes.byref(c), _ptr(S), _ptr(perm), _ptr(state), n_slots, _ptr(slot_idx),
-                                     S.shape[0], _stream(stream)), "damp_quantize_state")
+    B = S.shape[0]
+    try:
+        fits = (_fits_pool(torch, layout, state, perm, num_slots, B, slot_idx)
+                and _fit(S, (B, layout.heads_of_operands, layout.d_k, layout.d_v), torch.float32)
+                and (slot_idx is None or _fit(slot_idx, (B,), torch.int32)))
+    except (AttributeError, IndexError, TypeError):  # a missing tensor, or one of another kind
+        fits = False
+    if fits:
+        n_slots = state.shape[0] if num_slots is None else int(num_slots)
+    else:
+        n_slots = _want_pool(layout, state, num_slots)
+        _want_batch(slot_idx, B, n_slots)
+        _want("S", S, (B, layout.heads_of_operands, layout.d_k, layout.d_v), dtype=torch.float32)
+        _want("perm", perm, (layout.num_heads, layout.d_k), dtype=torch.uint8)
+        for n, t in (("S", S), ("perm", perm), ("state", state), ("slot_idx", slot_idx)):
+            _cuda_contig(n, t)
+    _check(lib().damp_quantize_state(_cptr(layout), S.data_ptr(), _addr(perm), state.data_ptr(), n_slots,
+                                     _addr(slot_idx), B, _raw_stream(torch, stream)), "damp_quantize_state")
 
 
 def dequantize_state(layout, state, perm, batch=None, S=None, slot_idx=None, num_slots=None, stream=None):
@@ -468,7 +578,10 @@ def dequantize_state(layout, state, perm, batch=None, S=None, slot_idx=None, num
     for n, t in (("S", S), ("perm", perm), ("state", state), ("slot_idx", slot_idx)):
         _cuda_contig(n, t)
     if S is None:
-        S = torch.zeros((B, layout.heads_of_operands, layout.d_k, layout.d_v), dtype=torch.float32, device=state.device)
+        # rows of a slot outside the pool or of another group's heads stay zero; without slot
+        # indices and a head map the call writes every row
+        alloc = torch.empty if slot_idx is None and layout.head_map is None else torch.zeros
+        S = alloc((B, layout.heads_of_operands, layout.d_k, layout.d_v), dtype=torch.float32, device=state.device)
     c = layout.c()
     _check(lib().damp_dequantize_state(ctypes.byref(c), _ptr(state), n_slots, _ptr(slot_idx), B,
                                        _ptr(perm), _ptr(S), _stream(stream)), "damp_dequantize_state")
