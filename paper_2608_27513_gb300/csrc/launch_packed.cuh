@@ -87,10 +87,10 @@ static cudaError_t packed_launch_shape(const StepArgs &a, uint32_t *status, Pack
         p.warp_smem = p.stage0_off + p.nstage * p.stage_bytes;
     }
     if (warps * p.warp_smem > smem_cap) return cudaErrorInvalidConfiguration;
-    const int64_t want = (p.total_tiles + warps - 1) / warps;
     out->p = p;
     out->warps = warps;
-    out->grid = (int)std::min<int64_t>(std::max<int64_t>(want, 1), (int64_t)sm_count());
+    // fewer tiles than the grid has warps: still one CTA per SM, the tiles spread evenly over them
+    out->grid = (int)std::min<int64_t>(std::max<int64_t>(p.total_tiles, 1), (int64_t)sm_count());
     out->smem = p.warp_smem * warps;
     return cudaSuccess;
 }
@@ -224,8 +224,7 @@ static cudaError_t launch_packed2_impl(const StepArgs &a1, const StepArgs &a2, c
     const int smem = ws * kPackedWarps;
     if (smem > max_smem_per_block()) return cudaErrorNotSupported;
     if ((e = ensure_smem_limit(reinterpret_cast<const void *>(kern), smem)) != cudaSuccess) return e;
-    const int grid = (int)std::min<int64_t>(std::max<int64_t>((std::max(t1, t2) + kPackedWarps - 1) / kPackedWarps, 1),
-                                            (int64_t)sm_count());
+    const int grid = (int)std::min<int64_t>(std::max(t1, t2), (int64_t)sm_count());
     kern<<<grid, 32 * kPackedWarps, smem, stream>>>(s1.p, s2.p);
     return cudaGetLastError();
 }

@@ -36,8 +36,7 @@ static cudaError_t launch_prefill_cg(const PrefillParams &p0, const StepArgs &a,
     int warps = kPrefillWarps;
     while (warps > 1 && warps * warp_smem > max_smem_per_block()) --warps;
     if (warps * warp_smem > max_smem_per_block()) return cudaErrorInvalidValue;
-    const int64_t want = (p.total_tiles + warps - 1) / warps;
-    const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count());
+    const int grid = (int)std::min<int64_t>(p.total_tiles, (int64_t)sm_count());
     const int smem = warp_smem * warps;
     void (*kern)(PrefillParams) = nullptr;
     if (a.dk == 64) kern = a.in_bf16 ? prefill_cg_kernel<64, KDA, HAD, true> : prefill_cg_kernel<64, KDA, HAD, false>;
@@ -106,12 +105,11 @@ static cudaError_t launch_prefill_impl(const StepArgs &a, cudaStream_t stream, u
         if (V > 4) return cudaErrorInvalidValue;
         extra = (warps / 4) * 2 * 4 * 128 * 4;  // per group: two buffers of [4 blocks][128 rows]
         if (warps * warp_smem + extra > max_smem_per_block()) return cudaErrorInvalidValue;
-        const int64_t units = p.total_tiles / V;
-        want = (units + warps / 4 - 1) / (warps / 4);
+        want = p.total_tiles / V;
     } else {
         while (warps > 1 && warps * warp_smem > max_smem_per_block()) --warps;
         if (warps * warp_smem > max_smem_per_block()) return cudaErrorInvalidValue;
-        want = (p.total_tiles + warps - 1) / warps;
+        want = p.total_tiles;
     }
     p.amax_off = warps * warp_smem;
     const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count());

@@ -56,8 +56,8 @@ static cudaError_t launch_quad_rowabs_impl(const StepArgs &a, cudaStream_t strea
     if (units == 0) return cudaSuccess;
     cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(kern), smem);
     if (e != cudaSuccess) return e;
-    // one CTA (two quads) per SM, fewer when there are fewer units than quads
-    const int grid = (int)std::min<int64_t>((units + kQfrWarps / 4 - 1) / (kQfrWarps / 4), (int64_t)sm_count());
+    // one CTA (two quads) per SM, fewer when there are fewer units than SMs
+    const int grid = (int)std::min<int64_t>(units, (int64_t)sm_count());
     kern<<<grid, 32 * kQfrWarps, smem, stream>>>(p);
     return cudaGetLastError();
 }

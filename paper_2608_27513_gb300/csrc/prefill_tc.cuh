@@ -60,7 +60,9 @@ constexpr int kSmScal = 181248; // a, beta, gamma, f_C. (64 floats each), pi, g,
 constexpr int kTcRowL = 68;     // floats per row of L'^T
 constexpr int kTcRowY = 132;    // floats per row of Y / U
 constexpr int kTcRowV = 272;    // bytes per row of v
-constexpr int kTcSmem = kSmScal + 1472;
+constexpr int kTcMaxSort = 512;  // batch rows up to which a ragged chunk's units are ordered by length
+constexpr int kSmOrder = kSmScal + 1472;
+constexpr int kTcSmem = kSmOrder + 2 * kTcMaxSort;
 constexpr int kTcMaxRec = 8192; // largest record (d_k = 128): four fit in [kSmRec, kSmV)
 __host__ __device__ constexpr int tc_rec_stride(int rec_bytes) { return (rec_bytes + 127) & ~127; }
 
@@ -121,6 +123,53 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const float (&v)[32]) {
                  : "memory");
 }
 
+// N = 8, 16 or 32 consecutive columns
+template <int N>
+__device__ __forceinline__ void tc_ldn(uint32_t taddr, float (&v)[N]) {
+    static_assert(N == 8 || N == 16 || N == 32, "columns per access");
+    if constexpr (N == 32) {
+        tc_ld32(taddr, v);
+    } else {
+        uint32_t r[N];
+        if constexpr (N == 16)
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+                         "tcgen05.wait::ld.sync.aligned;"
+                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                         : "r"(taddr)
+                         : "memory");
+        else
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                         "tcgen05.wait::ld.sync.aligned;"
+                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                         : "r"(taddr)
+                         : "memory");
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = __uint_as_float(r[i]);
+    }
+}
+template <int N>
+__device__ __forceinline__ void tc_stn(uint32_t taddr, const float (&v)[N]) {
+    static_assert(N == 8 || N == 16 || N == 32, "columns per access");
+    if constexpr (N == 32) {
+        tc_st32(taddr, v);
+    } else if constexpr (N == 16) {
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
+                     "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+                     "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
+                     "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
+                     "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
+                     "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
+                     : "memory");
+    } else {
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n"
+                     "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+                     "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
+                     "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
+                     : "memory");
+    }
+}
+
 // x = hi + mid + lo as bf16 parts (each the round-to-nearest of what is left), two
 // values per 32-bit word (a in the low half)
 __device__ __forceinline__ void split3_pair(float a, float b, uint32_t &h, uint32_t &m, uint32_t &l) {
@@ -178,17 +227,16 @@ __device__ __forceinline__ uint32_t tc_k64_off(int row, int k) {
     return (uint32_t)(row >> 3) * 1024u + (uint32_t)(k >> 3) * 128u + (uint32_t)(row & 7) * 16u + (uint32_t)(k & 7) * 2u;
 }
 
-// The record rows of a (slot, head) (four value-block records at `recs`, `rstride` apart
-// in shared memory) reconstructed into tensor-memory lane u = record row, the value blocks
-// of part `part` of NQ (4 / NQ blocks each): FP32 at the natural scale, FP16 rows taken
+// The record rows of a (slot, head) (value-block records at `recs`, `rstride` apart in shared
+// memory) reconstructed into tensor-memory lane u = record row, blocks ca .. cb - 1: FP32 at the natural scale, FP16 rows taken
 // into the H_32 domain with the H_32 formats (where the low tier's codes already are).
-template <int FMT, int NQ>
-__device__ __forceinline__ void tc_reconstruct(const PrefillParams &p, uint32_t recs, int rstride, int u, int part,
+template <int FMT>
+__device__ __forceinline__ void tc_reconstruct(const PrefillParams &p, uint32_t recs, int rstride, int u, int ca, int cb,
                                                uint32_t tS) {
     constexpr bool HAD = fmt_had(FMT);
     const int K = p.K, lo = 128 - K;
 #pragma unroll 1
-    for (int c = part * (4 / NQ); c < (part + 1) * (4 / NQ); ++c) {
+    for (int c = ca; c < cb; ++c) {
         const uint32_t rec = recs + (uint32_t)(c * rstride);
         float2 y[16];
         if (u < K) {
@@ -227,7 +275,8 @@ __device__ __forceinline__ void bar_sync(int id, int threads) {
 
 // U = L^-1 Y by forward substitution, in place: yu addresses row 0 of Y (rows kTcRowY floats
 // apart), lt the rows of L'^T (L' = L - I, kTcRowL floats apart).  Warp w of NW owns the rows
-// RW w .. RW w + RW - 1 (RW = 64 / NW) of all 128 columns, lane l the columns 4 l .. 4 l + 3,
+// RW w .. RW w + RW - 1 (RW = 64 / NW) of all 32 NV columns, lane l the columns 4 l .. 4 l + 3
+// (l mod 8 NV: with fewer than 128 columns lanes repeat one another's work, their loads merge),
 // in registers.  Step j: warp j solves its rows among themselves and stores them; the warps
 // after it take them out of their own rows, each value of L' and of U loaded once per RW x 4
 // tile.  Every element subtracts its products in ascending row order.  Every thread of the CTA
@@ -235,12 +284,12 @@ __device__ __forceinline__ void bar_sync(int id, int threads) {
 // cycles with 16 warps at 128 bytes a cycle): a 64-token KDA piece 8400 -> 6000 cycles against
 // a thread per column and quarter of the rows, whose every 16-byte load of L' fed four products
 // (on 8 of the 16 warps: 8000); the GDN chunk of B = 256 x 64 tokens 934 -> 878 us.
-template <int NW>
+template <int NW, int NV>
 __device__ __forceinline__ void tc_solve(uint32_t yu, uint32_t lt, int warp, int lane) {
     constexpr int RW = kTcC / NW;  // 4 or 8
     static_assert(RW % 4 == 0, "a warp's rows of L'^T are read in 16-byte vectors");
     const int r0 = RW * warp;
-    const uint32_t col = yu + (uint32_t)(16 * lane), lrow = lt + (uint32_t)(4 * r0);
+    const uint32_t col = yu + (uint32_t)(16 * (lane & (8 * NV - 1))), lrow = lt + (uint32_t)(4 * r0);
     float2 acc[RW][2];
     auto row = [&](int r, float2 (&v)[2]) {
         const uint4 w = lds128(col + (uint32_t)(r * kTcRowY * 4));
@@ -298,17 +347,17 @@ __device__ __forceinline__ void tc_solve(uint32_t yu, uint32_t lt, int warp, int
     if (warp < NW - 1) bar_arrive(1 + (warp & 1), 32 * (NW - warp));
 }
 
-// The chunk-final state (tensor-memory lane u = record row u, the value blocks of part
-// `part` of NQ) into the records at grec0 in place: FP16 rows back to the natural domain
+// The chunk-final state (tensor-memory lane u = record row u, blocks ca .. cb - 1) into the
+// records at grec0 in place: FP16 rows back to the natural domain
 // and rounded once, low-tier rows requantized (the affine formats at the working scale
 // 2^-39, FP8 in the natural domain).  Warps holding FP16 rows store them warp-collectively.
-template <int FMT, int NQ>
-__device__ __forceinline__ void tc_requantize(const PrefillParams &p, uint8_t *grec0, int u, int part, int lane,
+template <int FMT>
+__device__ __forceinline__ void tc_requantize(const PrefillParams &p, uint8_t *grec0, int u, int ca, int cb, int lane,
                                               uint32_t tS) {
     constexpr bool HAD = fmt_had(FMT);
     const int K = p.K, lo = 128 - K;
 #pragma unroll 1
-    for (int c = part * (4 / NQ); c < (part + 1) * (4 / NQ); ++c) {
+    for (int c = ca; c < cb; ++c) {
         float v[32];
         tc_ld32(tS + 32 * c, v);
         uint8_t *const grec = grec0 + (int64_t)c * p.rec_bytes;
@@ -359,6 +408,63 @@ __device__ __forceinline__ void tc_requantize(const PrefillParams &p, uint8_t *g
     }
 }
 
+// Which units a CTA of the persistent grid takes: in round r the units at position r * grid +
+// blk of the order, in odd rounds from the other end (r * grid + grid - 1 - blk).  The order is
+// head by head through the batch rows, and for a ragged chunk through the rows by falling length
+// (up to kTcMaxSort rows: `order`, uint16 in shared memory, filled by tc_sort_rows), so that the
+// CTAs with the longest units get the shortest ones next.  KDA, 13 rows of up to 133 tokens x 32
+// heads (416 units on 152 SMs): 176 us in batch order, 134 us so.
+__device__ __forceinline__ void tc_sort_rows(const PrefillParams &p, uint32_t order) {
+    for (int b = threadIdx.x; b < p.batch; b += blockDim.x) {
+        const int len = p.lengths[b];
+        int rank = 0;
+        for (int c = 0; c < p.batch; ++c) {
+            const int other = p.lengths[c];
+            rank += other > len || (other == len && c < b);
+        }
+        asm volatile("st.shared.u16 [%0], %1;" ::"r"(order + 2 * rank), "h"((unsigned short)b) : "memory");
+    }
+}
+struct TcUnit {
+    int64_t slot;
+    int b, h, mh, hq, Tb;  // batch row, held, model and q/k head, tokens
+    int c0;                // first value block
+    bool ok;               // false past the CTA's last unit
+};
+// A unit is NV of a (slot, head)'s four value blocks (the closed form's value columns are
+// independent).  The fewer, the more of the work that does not depend on the values is repeated,
+// but with few (slot, head) pairs the SMs would be idle: NV = 1 or 2 where all the units then still
+// run at once (KDA, 32 heads: one prompt of 2048 tokens 737 us with NV = 4, 643 with 1; two of 500
+// tokens 190 / 168 with 2).
+__host__ __device__ constexpr int tc_nv(int64_t pairs, int sms) { return 4 * pairs <= sms ? 1 : 2 * pairs <= sms ? 2 : 4; }
+// The CTA's next unit with work at or after round `round` (left after it); units without work are
+// skipped, their status bits collected.
+template <int NV>
+__device__ __forceinline__ TcUnit tc_next_unit(const PrefillParams &p, int64_t &round, bool sorted, uint32_t order,
+                                               bool &bad_slot, bool &bad_head) {
+    TcUnit n{0, 0, 0, 0, 0, 0, 0, false};
+    constexpr int S = 4 / NV;
+    const int HS = p.H * S;
+    const int64_t units = (int64_t)p.batch * HS, grid = gridDim.x;
+    for (; round * grid < units && !n.ok; ++round) {
+        const int64_t at = round * grid + ((round & 1) ? grid - 1 - blockIdx.x : blockIdx.x);
+        if (at >= units) continue;
+        const int r = (int)(at / HS), hs = (int)(at - (int64_t)r * HS);
+        n.h = hs / S;
+        n.c0 = NV * (hs - n.h * S);
+        n.b = sorted ? (int)lds_u16(order + 2 * r) : r;
+        n.mh = p.head_map ? p.head_map[n.h] : n.h;
+        n.slot = p.slot_idx ? (int64_t)p.slot_idx[n.b] : (int64_t)n.b;
+        n.Tb = p.lengths ? min(max(p.lengths[n.b], 0), p.T) : p.T;
+        const bool slot_ok = n.slot >= 0 && n.slot < p.num_slots, head_ok = n.mh >= 0 && n.mh < p.Hm;
+        bad_slot |= !slot_ok;
+        bad_head |= !head_ok;
+        n.ok = slot_ok && head_ok && n.Tb > 0;
+        n.hq = (int)(((int64_t)n.mh * p.Hqk) / p.Hm);
+    }
+    return n;
+}
+
 // One CTA of kTcThreads threads per (slot, head) unit at a time (persistent over units);
 // d_k = d_v = 128, bf16 q/k/v, low tier FMT (UINT8 or UINT4 affine, with or without H_32;
 // the launchers also instantiate no FP8 or row-absmax kernel).  Thread (row, half):
@@ -372,7 +478,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = tid & 127, half = tid >> 7;
     const uint32_t sb = smem_u32(smem);
-    const int H = p.H, T = p.T, Hm = p.Hm;
+    const int T = p.T, Hm = p.Hm;
     const int rec_bytes = p.rec_bytes, rstride = tc_rec_stride(rec_bytes);
     const uint32_t scal = sb + (uint32_t)kSmScal;
     const uint32_t s_a = scal, s_beta = scal + 256, s_gam = scal + 512, s_rev = scal + 768, s_perm = scal + 1024;
@@ -388,6 +494,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
         mbar_init(bar_mma, 1);
         fence_mbar_init();
     }
+    if (p.lengths && p.batch <= kTcMaxSort) tc_sort_rows(p, sb + (uint32_t)kSmOrder);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -398,35 +505,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
     uint32_t ph_rec = 0, ph_mma = 0;
     bool bad_slot = false, bad_head = false, timed_out = false;
     bool rec_pending = false, mma_pending = false;  // a copy / a product in flight
-    const int64_t units = (int64_t)p.batch * H;
-    // a (slot, head) unit that has work: its batch row, held and model head, slot and length
-    struct Unit {
-        int64_t unit, slot;
-        int b, h, mh, hq, Tb;
-    };
-    // the first unit at or after u (stepping by the grid) with work; unit == units if none
-    // (units without work are skipped here, once each, with their status bits)
-    auto next_unit = [&](int64_t u) -> Unit {
-        Unit n{units, 0, 0, 0, 0, 0, 0};
-        for (; u < units; u += gridDim.x) {
-            const int b = (int)(u / H), h = (int)(u - (int64_t)b * H);
-            const int mh = p.head_map ? p.head_map[h] : h;
-            const int64_t slot = p.slot_idx ? (int64_t)p.slot_idx[b] : (int64_t)b;
-            const int Tb = p.lengths ? min(max(p.lengths[b], 0), T) : T;
-            const bool slot_ok = slot >= 0 && slot < p.num_slots, head_ok = mh >= 0 && mh < Hm;
-            bad_slot |= !slot_ok;
-            bad_head |= !head_ok;
-            if (slot_ok && head_ok && Tb > 0) {
-                n = Unit{u, slot, b, h, mh, (int)(((int64_t)mh * p.Hqk) / Hm), Tb};
-                break;
-            }
-        }
-        return n;
-    };
-    auto rec_of = [&](const Unit &n) { return p.state + n.slot * p.slot_bytes + (int64_t)(n.h * 4) * rec_bytes; };
+    int64_t round = 0;
+    const bool sorted = p.lengths && p.batch <= kTcMaxSort;
+    auto next_unit = [&]() { return tc_next_unit<4>(p, round, sorted, sb + (uint32_t)kSmOrder, bad_slot, bad_head); };
+    auto rec_of = [&](const TcUnit &n) { return p.state + n.slot * p.slot_bytes + (int64_t)(n.h * 4) * rec_bytes; };
     // [K; Q] (bf16, natural channel order, K-major), v, g and beta of unit n's piece at p0
     // (cp.async; a masked token is zero, neither decays nor updates)
-    auto load_piece = [&](const Unit &n, int p0) {
+    auto load_piece = [&](const TcUnit &n, int p0) {
         const int nt = min(kTcC, n.Tb - p0);
 #pragma unroll 1
         for (int i = tid; i < 2048; i += kTcThreads) {
@@ -464,7 +549,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
     };
     // unit n's four records (bulk copies), pi and first piece: issued one unit ahead, so
     // that they land while the previous unit finishes (every area they write is free then)
-    auto prefetch = [&](const Unit &n) {
+    auto prefetch = [&](const TcUnit &n) {
         if (tid == 0) {
             fence_proxy_async_smem();
             mbar_arrive_expect_tx(bar_rec, (uint32_t)(4 * rec_bytes));
@@ -478,12 +563,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
         rec_pending = true;
     };
 
-    Unit cur = next_unit(blockIdx.x);
-    if (cur.unit < units) prefetch(cur);
-    while (cur.unit < units) {
+    TcUnit cur = next_unit();
+    if (cur.ok) prefetch(cur);
+    while (cur.ok) {
         const int b = cur.b, Tb = cur.Tb, mh = cur.mh;
         uint8_t *const grec0 = rec_of(cur);
-        const Unit nxt = next_unit(cur.unit + gridDim.x);  // its loads overlap this unit's work
+        const TcUnit nxt = next_unit();  // its loads overlap this unit's work
         if (!tc_wait_all(bar_rec, ph_rec)) {
             timed_out = true;
             break;
@@ -493,7 +578,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
 
         // ---- S_0: record row u = row, reconstructed (FP32, natural scale, transformed domain
         //      with H_32) into tensor-memory lane u; this half's two value blocks ----
-        tc_reconstruct<FMT, 2>(p, sb + (uint32_t)kSmRec, rstride, row, half, tS);
+        tc_reconstruct<FMT>(p, sb + (uint32_t)kSmRec, rstride, row, 2 * half, 2 * half + 2, tS);
 
 #pragma unroll 1
         for (int p0 = 0; p0 < Tb; p0 += kTcC) {
@@ -683,7 +768,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
             }
             __syncthreads();
             // ---- U = L^-1 Y by forward substitution, in place ----
-            tc_solve<kTcThreads / 32>(sb + (uint32_t)kSmYU, sb + (uint32_t)kSmLP, warp, lane);
+            tc_solve<kTcThreads / 32, 4>(sb + (uint32_t)kSmYU, sb + (uint32_t)kSmLP, warp, lane);
             __syncthreads();
             // ---- U (half 0) and f_C. U (half 1) as three bf16 parts, K-major (value columns n x
             //      tokens s) ----
@@ -730,7 +815,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
             }
             ph_mma ^= 1u;
             tc_fence_after();
-            if (p0 + kTcC >= Tb && nxt.unit < units) prefetch(nxt);  // the next unit's loads overlap this one's tail
+            if (p0 + kTcC >= Tb && nxt.ok) prefetch(nxt);  // the next unit's loads overlap this one's tail
             // ---- o_t = H (gamma_t P_t + (M U)_t) (lanes 64 + t, this half's value blocks) ----
             if (row >= 64) {
                 const int t = row - 64;
@@ -755,7 +840,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
         if (timed_out) break;
         // ---- the chunk-final state (tensor-memory lane u = record row u, this half's value
         //      blocks) into the record in place ----
-        tc_requantize<FMT, 2>(p, grec0, row, half, lane, tS);
+        tc_requantize<FMT>(p, grec0, row, 2 * half, 2 * half + 2, lane, tS);
         cur = nxt;
     }
     // a copy or a product that did not complete in time gets one more bounded wait before

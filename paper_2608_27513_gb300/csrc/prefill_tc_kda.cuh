@@ -49,7 +49,8 @@ constexpr int kKdAO = 152576;       // [.; M]: three bf16 parts, K-major (128 ro
 constexpr int kKdYU = 0;            // Y, then U: 64 rows of kTcRowY FP32
 __host__ __device__ constexpr int kd_bu(int part) { return part == 2 ? 135168 : 16384 * part; }  // U: three bf16 parts, K-major (value columns x tokens)
 constexpr int kKdScal = 208896;     // beta, pi, gamma_m, xi_C, mbarriers, TMEM address
-constexpr int kKdSmem = kKdScal + 2048;
+constexpr int kKdOrder = kKdScal + 2048;
+constexpr int kKdSmem = kKdOrder + 2 * kTcMaxSort;
 constexpr int kKdMaxRec = 8192;     // four records fit in [kKdRec, kKdZ)
 constexpr float kKdMaxLog = 85.0f;  // largest log-range of xi on either side of the reference token
 constexpr int kKdThreads = 512;     // four threads per tensor-memory lane (warps w, w + 4, w + 8, w + 12)
@@ -58,15 +59,17 @@ constexpr int kKdThreads = 512;     // four threads per tensor-memory lane (warp
 // d_k = d_v = 128, bf16 q/k/v, low tier FMT (UINT8 or UINT4 affine, with or without H_32).
 // Thread (row, quarter qq): row = tensor-memory lane (warps w, w + 4, w + 8 and w + 12
 // reach the same lanes); the quarters split a row's value blocks (one each) or a phase's tasks.
-template <int FMT>
+template <int FMT, int NV>
 __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const PrefillParams p) {
     static_assert(FMT != kFmtS8Row, "the row-absmax format shares a row scale over the value blocks");
     constexpr bool HAD = fmt_had(FMT);
+    constexpr int NC = 32 * NV, CQ = NC / 4;  // value columns of a unit, and of a quarter of its threads
+    constexpr uint32_t kIdWPn = tc_idesc(NC, false, true), kIdOn = tc_idesc(NC, false, false);
     extern __shared__ __align__(128) uint8_t smem[];  // descriptors need 16-byte alignment (no swizzle)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = tid & 127, qq = tid >> 7;
     const uint32_t sb = smem_u32(smem);
-    const int H = p.H, T = p.T, Hm = p.Hm;
+    const int T = p.T, Hm = p.Hm;
     const int rec_bytes = p.rec_bytes, rstride = tc_rec_stride(rec_bytes);
     const uint32_t scal = sb + (uint32_t)kKdScal;
     const uint32_t s_beta = scal, s_perm = scal + 256, s_gm = scal + 384, s_xiC = scal + 1408;
@@ -83,6 +86,7 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         mbar_init(bar_mma, 1);
         fence_mbar_init();
     }
+    if (p.lengths && p.batch <= kTcMaxSort) tc_sort_rows(p, sb + (uint32_t)kKdOrder);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -93,33 +97,13 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
     uint32_t ph_rec = 0, ph_mma = 0;
     bool bad_slot = false, bad_head = false, timed_out = false;
     bool rec_pending = false, mma_pending = false;  // a copy / a product in flight
-    const int64_t units = (int64_t)p.batch * H;
-    struct Unit {
-        int64_t unit, slot;
-        int b, h, mh, hq, Tb;
-    };
-    // the first unit at or after u (stepping by the grid) with work; unit == units if none
-    auto next_unit = [&](int64_t u) -> Unit {
-        Unit n{units, 0, 0, 0, 0, 0, 0};
-        for (; u < units; u += gridDim.x) {
-            const int b = (int)(u / H), h = (int)(u - (int64_t)b * H);
-            const int mh = p.head_map ? p.head_map[h] : h;
-            const int64_t slot = p.slot_idx ? (int64_t)p.slot_idx[b] : (int64_t)b;
-            const int Tb = p.lengths ? min(max(p.lengths[b], 0), T) : T;
-            const bool slot_ok = slot >= 0 && slot < p.num_slots, head_ok = mh >= 0 && mh < Hm;
-            bad_slot |= !slot_ok;
-            bad_head |= !head_ok;
-            if (slot_ok && head_ok && Tb > 0) {
-                n = Unit{u, slot, b, h, mh, (int)(((int64_t)mh * p.Hqk) / Hm), Tb};
-                break;
-            }
-        }
-        return n;
-    };
-    auto rec_of = [&](const Unit &n) { return p.state + n.slot * p.slot_bytes + (int64_t)(n.h * 4) * rec_bytes; };
+    int64_t round = 0;
+    const bool sorted = p.lengths && p.batch <= kTcMaxSort;
+    auto next_unit = [&]() { return tc_next_unit<NV>(p, round, sorted, sb + (uint32_t)kKdOrder, bad_slot, bad_head); };
+    auto rec_of = [&](const TcUnit &n) { return p.state + n.slot * p.slot_bytes + (int64_t)(n.h * 4 + n.c0) * rec_bytes; };
     // g, v and beta of unit n's tokens p0 .. p0 + 63 (cp.async; rows past the row's length are
     // zero), issued while the products of the piece before run
-    auto load_gv = [&](const Unit &n, int p0) {
+    auto load_gv = [&](const TcUnit &n, int p0) {
         const int nl = min(kTcC, n.Tb - p0);
 #pragma unroll 1
         for (int i = tid; i < 2048; i += kKdThreads) {  // g: 64 rows of 32 chunks
@@ -147,7 +131,7 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         cp_async_commit();
     };
     // its k and q (needed after the decay ratios), once the products that read U are done
-    auto load_kq = [&](const Unit &n, int p0) {
+    auto load_kq = [&](const TcUnit &n, int p0) {
         const int nl = min(kTcC, n.Tb - p0);
 #pragma unroll 1
         for (int i = tid; i < 2048; i += kKdThreads) {  // k rows 0..63, q rows 64..127: 16 chunks each
@@ -162,29 +146,29 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         cp_async_commit();
     };
     // unit n's records and pi, one unit ahead (their copies join load_kq's group)
-    auto load_records = [&](const Unit &n) {
+    auto load_records = [&](const TcUnit &n) {
         if (tid == 0) {
             fence_proxy_async_smem();
-            mbar_arrive_expect_tx(bar_rec, (uint32_t)(4 * rec_bytes));
+            mbar_arrive_expect_tx(bar_rec, (uint32_t)(NV * rec_bytes));
             uint8_t *const g0 = rec_of(n);
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
+            for (int c = 0; c < NV; ++c)
                 bulk_g2s(sb + (uint32_t)(kKdRec + c * rstride), g0 + (int64_t)c * rec_bytes, (uint32_t)rec_bytes, bar_rec);
         }
         if (tid < 8) cp_async16(s_perm + 16 * tid, p.perm + (int64_t)n.h * 128 + 16 * tid);
         rec_pending = true;
     };
 
-    Unit cur = next_unit(blockIdx.x);
-    if (cur.unit < units) {
+    TcUnit cur = next_unit();
+    if (cur.ok) {
         load_gv(cur, 0);
         load_records(cur);
         load_kq(cur, 0);
     }
-    while (cur.unit < units) {
+    while (cur.ok) {
         const int b = cur.b, Tb = cur.Tb, mh = cur.mh;
         uint8_t *const grec0 = rec_of(cur);
-        const Unit nxt = next_unit(cur.unit + gridDim.x);  // its loads overlap this unit's work
+        const TcUnit nxt = next_unit();  // its loads overlap this unit's work
         if (!tc_wait_all(bar_rec, ph_rec)) {
             timed_out = true;
             break;
@@ -192,8 +176,10 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         ph_rec ^= 1u;
         rec_pending = false;
         // ---- S_0: record row u = row into tensor-memory lane u (this quarter's value block) ----
-        tc_reconstruct<FMT, 4>(p, sb + (uint32_t)kKdRec, rstride, row, qq, tS);
-        __syncthreads();  // the records are read: the first piece's operands go over them
+        if (qq < NV) tc_reconstruct<FMT>(p, sb + (uint32_t)kKdRec, rstride, row, qq, qq + 1, tS);
+        tc_fence_before();  // (with NV < 4 the state's columns are split differently below)
+        __syncthreads();    // the records are read: the first piece's operands go over them
+        tc_fence_after();
 
         int p0 = 0;
 #pragma unroll 1
@@ -316,17 +302,14 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
                     const int ch = (int)(lds_u8(s_perm + row) & 127u);
                     const bool mine = (ch >> 6) == hh;
                     const float gmc = ldsf(s_gm + 4 * ch);
-                    {
-                        const int c = qq;
-                        float v[32];
-                        tc_ld32(tS + 32 * c, v);  // every lane: warp-collective
-                        if (mine) {
+                    float v[CQ];
+                    tc_ldn<CQ>(tS + CQ * qq, v);  // every lane: warp-collective
+                    if (mine) {
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) v[i] *= gmc;
+                        for (int i = 0; i < CQ; ++i) v[i] *= gmc;
 #pragma unroll
-                            for (int j8 = 0; j8 < 4; ++j8)
-                                split3_store8(sb + kKdB1 + tc_mn_off(32 * c + 8 * j8, ch & 63, 2048), 16384, v + 8 * j8);
-                        }
+                        for (int j8 = 0; j8 < CQ / 8; ++j8)
+                            split3_store8(sb + kKdB1 + tc_mn_off(CQ * qq + 8 * j8, ch & 63, 2048), 16384, v + 8 * j8);
                     }
                 }
                 fence_proxy_async_smem();
@@ -340,7 +323,7 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
                             tc_mma(tmem + kColWP, tc_desc(sb + kKdX + 16384 * pa[q] + 256 * ks, 128, 1024),
-                                   tc_desc(sb + kKdB1 + 16384 * pb[q] + 4096 * ks, 2048, 128), kIdWP, (hh | q | ks) != 0);
+                                   tc_desc(sb + kKdB1 + 16384 * pb[q] + 4096 * ks, 2048, 128), kIdWPn, (hh | q | ks) != 0);
 #pragma unroll
                     for (int q = 0; q < 6; ++q)
 #pragma unroll
@@ -402,21 +385,18 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
             {  // gamma_C S_0 = gamma_m xi_C S_0 (per channel; the state product accumulates onto it)
                 const uint32_t ch = lds_u8(s_perm + row) & 127u;
                 const float gc = ldsf(s_gm + 4u * ch) * ldsf(s_xiC + 4u * ch);
-                {
-                    const int c = qq;
-                    float v[32];
-                    tc_ld32(tS + 32 * c, v);
+                float v[CQ];
+                tc_ldn<CQ>(tS + CQ * qq, v);
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] *= gc;
-                    tc_st32(tS + 32 * c, v);
-                }
+                for (int i = 0; i < CQ; ++i) v[i] *= gc;
+                tc_stn<CQ>(tS + CQ * qq, v);
             }
             __syncthreads();  // K and Xi are read: Y goes over them
             // ---- Y = diag(beta) (v~ - W), FP32 rows (this quarter's value block) ----
-            if (row < 64) {
+            if (row < 64 && qq < NV) {
                 const int t = row;
                 const float bt = ldsf(s_beta + 4 * t);
-                const uint32_t vrow = sb + (uint32_t)(kKdV + t * kTcRowV), yrow = sb + (uint32_t)(kKdYU + t * kTcRowY * 4);
+                const uint32_t vrow = sb + (uint32_t)(kKdV + t * kTcRowV + 64 * cur.c0), yrow = sb + (uint32_t)(kKdYU + t * kTcRowY * 4);
                 {
                     const int c = qq;
                     float w[32];
@@ -444,19 +424,23 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
             // g, v and beta are read: the next piece's go over them
             const bool last = p0 + nt >= Tb;
             if (!last) load_gv(cur, p0 + nt);
-            else if (nxt.unit < units) load_gv(nxt, 0);
+            else if (nxt.ok) load_gv(nxt, 0);
             // ---- U = L^-1 Y, in place ----
-            tc_solve<kKdThreads / 32>(sb + (uint32_t)kKdYU, sb + (uint32_t)kKdLP, warp, lane);
+            tc_solve<kKdThreads / 32, NV>(sb + (uint32_t)kKdYU, sb + (uint32_t)kKdLP, warp, lane);
             __syncthreads();
             // ---- U as three bf16 parts, K-major (value columns n x tokens s): tokens 16 qq .. + 15 ----
             {
                 const uint32_t col = sb + (uint32_t)(kKdYU + 4 * row);
                 float uc[16];
+                if (row < NC) {
 #pragma unroll
-                for (int t = 0; t < 16; ++t) uc[t] = ldsf(col + (uint32_t)((16 * qq + t) * kTcRowY * 4));
+                    for (int t = 0; t < 16; ++t) uc[t] = ldsf(col + (uint32_t)((16 * qq + t) * kTcRowY * 4));
+                }
                 __syncthreads();  // every column is read: the parts go over Y / U
+                if (row < NC) {
 #pragma unroll
-                for (int g = 0; g < 2; ++g) split3_store8(sb + tc_k64_off(row, 16 * qq + 8 * g), kd_bu(1), kd_bu(2), uc + 8 * g);
+                    for (int g = 0; g < 2; ++g) split3_store8(sb + tc_k64_off(row, 16 * qq + 8 * g), kd_bu(1), kd_bu(2), uc + 8 * g);
+                }
             }
             fence_proxy_async_smem();
             tc_fence_before();
@@ -470,13 +454,13 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
                         tc_mma(tmem + kColWP, tc_desc(sb + kKdAO + 16384 * pa[q] + 256 * ks, 128, 1024),
-                               tc_desc(sb + kd_bu(pb[q]) + 256 * ks, 128, 1024), kIdO, 1u);
+                               tc_desc(sb + kd_bu(pb[q]) + 256 * ks, 128, 1024), kIdOn, 1u);
 #pragma unroll
                 for (int q = 0; q < 6; ++q)
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
                         tc_mma(tmem + kColS, tc_desc(sb + kKdA3 + 16384 * pa[q] + 256 * ks, 128, 1024),
-                               tc_desc(sb + kd_bu(pb[q]) + 256 * ks, 128, 1024), kIdO, 1u);
+                               tc_desc(sb + kd_bu(pb[q]) + 256 * ks, 128, 1024), kIdOn, 1u);
                 tc_commit(bar_mma);
             }
             if (!tc_wait_all(bar_mma, ph_mma)) {
@@ -488,14 +472,14 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
             // the next piece's or unit's loads overlap this one's tail
             if (!last) {
                 load_kq(cur, p0 + nt);
-            } else if (nxt.unit < units) {
+            } else if (nxt.ok) {
                 load_records(nxt);
                 load_kq(nxt, 0);
             }
             // ---- o_t = H (P_t + (M U)_t) (lanes 64 + t, this quarter's value block) ----
-            if (row >= 64) {
+            if (row >= 64 && qq < NV) {
                 const int t = row - 64;
-                float *orow = p.o + (((int64_t)b * T + p0 + min(t, nt - 1)) * Hm + mh) * 128;
+                float *orow = p.o + (((int64_t)b * T + p0 + min(t, nt - 1)) * Hm + mh) * 128 + 32 * cur.c0;
                 {
                     const int c = qq;
                     float ov[32];
@@ -516,7 +500,7 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         }
         if (timed_out) break;
         // ---- the chunk-final state into the record in place ----
-        tc_requantize<FMT, 4>(p, grec0, row, qq, lane, tS);
+        if (qq < NV) tc_requantize<FMT>(p, grec0, row, qq, qq + 1, lane, tS);
         cur = nxt;
     }
     if (rec_pending) mbar_wait_bounded(bar_rec, ph_rec);

@@ -4,11 +4,14 @@ KDA, d_k = d_v = 128, bf16 q/k/v, chunks of at least 32 tokens (one or more piec
 to 64 tokens, ragged rows masked); the UINT8 and UINT4 low tiers.  KDA pieces are cut
 short where a channel's decay would leave FP32 on either side of the reference token."""
 import pytest
+import torch
 
+import paper_2608_27513_gb300 as damp
 import workloads as wl
 from tests.test_gpu_prefill import _built, _run  # noqa: F401  (module fixture and runner)
 
 pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
 
 
 def _gdn(name, batch, heads, qk_heads, k_hi, fmt=0, seed=31):
@@ -71,3 +74,36 @@ def test_kda_strong_decay_shortens_the_pieces(g_scale):
     channel): the pieces are cut to 32 tokens or fewer, down to single tokens, and the
     chunk still matches the per-token recurrence."""
     _run(_kda(f"tck_decay{int(g_scale)}", 1, 2, 2, 12, seed=45), 64, g_scale=g_scale)
+
+
+@pytest.mark.parametrize("kind", ["gdn", "kda"])
+@pytest.mark.parametrize("B,T", [(1, 40), (8, 70), (40, 130), (512, 32), (513, 33)])
+def test_ragged_batches_equal_their_rows_alone(kind, B, T):
+    """The units of a ragged chunk are taken by falling length (up to 512 rows), in rounds from both
+    ends of the order, KDA heads in one, two or four value parts by the number of pairs: every row, empty, full and equally long ones among them, gets what a call of
+    its own gives it, bit for bit, and rows past a length stay zero."""
+    H = 8
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(B)
+    n = lambda *s: torch.randn(*s, generator=gen, device=DEV)
+    unit = lambda x: (x / x.norm(dim=-1, keepdim=True)).bfloat16()
+    q, k, v = unit(n(B, T, H, 128)), unit(n(B, T, H, 128)), n(B, T, H, 128).bfloat16()
+    g = -torch.nn.functional.softplus(n(B, T, H) if kind == "gdn" else n(B, T, H, 128) - 3.0)
+    beta = torch.sigmoid(n(B, T, H))
+    lengths = torch.randint(0, T + 1, (B,), generator=gen, device=DEV, dtype=torch.int32)
+    lengths[B // 2] = T
+    lengths[: B // 4] = T // 2
+    L = damp.Layout(H, H, 128, 128, 16, 0)
+    perm = torch.stack([torch.randperm(128, generator=gen, device=DEV) for _ in range(H)]).to(torch.uint8)
+    pool = damp.new_state(L, B, DEV)
+    damp.quantize_state(L, 0.1 * n(B, H, 128, 128), perm, pool)
+    alone = pool.clone()
+    chunk = damp.kda_prefill_chunk if kind == "kda" else damp.gdn_prefill_chunk
+    o = chunk(L, pool, perm, q, k, v, g, beta, lengths=lengths)
+    for b in range(B):
+        ob = chunk(L, alone[b:b + 1], perm, q[b:b + 1], k[b:b + 1], v[b:b + 1], g[b:b + 1], beta[b:b + 1],
+                   lengths=lengths[b:b + 1].clone())
+        assert torch.equal(o[b:b + 1], ob)
+        assert not o[b, int(lengths[b]):].any()
+    assert torch.equal(pool, alone)
+    assert damp.device_status() == 0
