@@ -421,10 +421,6 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
                 }
             }
             __syncthreads();
-            // g, v and beta are read: the next piece's go over them
-            const bool last = p0 + nt >= Tb;
-            if (!last) load_gv(cur, p0 + nt);
-            else if (nxt.ok) load_gv(nxt, 0);
             // ---- U = L^-1 Y, in place ----
             tc_solve<kKdThreads / 32, NV>(sb + (uint32_t)kKdYU, sb + (uint32_t)kKdLP, warp, lane);
             __syncthreads();
@@ -463,6 +459,10 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
                                tc_desc(sb + kd_bu(pb[q]) + 256 * ks, 128, 1024), kIdOn, 1u);
                 tc_commit(bar_mma);
             }
+            // g, v and beta are read: the next piece's go over them while the products run
+            const bool last = p0 + nt >= Tb;
+            if (!last) load_gv(cur, p0 + nt);
+            else if (nxt.ok) load_gv(nxt, 0);
             if (!tc_wait_all(bar_mma, ph_mma)) {
                 timed_out = mma_pending = true;
                 break;
