@@ -17,8 +17,8 @@
 //
 // Measured (B = 64, H = 32, d = 128, GDN, 268 MB of state per step, more than L2): 46.9 us, 5.8
 // TB/s, bound by HBM; 49.6 us with one column per lane and each tile loaded, computed and
-// stored in turn.  A calibration run over 32 documents (KDA): ~22 us for one token (the 134 MB
-// that the states move through L2), 40 us for eight, 3.1 us per further token -- FP32
+// stored in turn.  A calibration run over 32 documents (KDA): ~20 us for one token (the 134 MB
+// that the states move through L2), 36 us for eight, 2.6 us per further token -- FP32
 // arithmetic (1.3 us at the FMA rate) and the operand loads, with two warps per scheduler.
 // With one launch per token the eight tokens between two samples took 165 us.
 #include "damp_common.cuh"
@@ -47,6 +47,16 @@ struct Fp32Params {
 constexpr int kFp32Warps = 4;
 constexpr int kFp32Ctas = 2;    // CTAs per SM: a third (168 registers a thread) spills, step 47 -> 54 us (below)
 constexpr int kFp32Tokens = 8;  // tokens staged at a time by a calibration run
+
+// A staged operand vector.  A run's loads keep their place in the program (one group of four rows
+// ahead of their use): left to the compiler, they are all moved to the front of the token, over the
+// registers that hold the state (170 bytes of spills; a 32 x 256 run 1805 us, so 1680).
+template <bool RUN>
+__device__ __forceinline__ float4 staged4(const float *p) {
+    if (!RUN) return *reinterpret_cast<const float4 *>(p);
+    const uint4 w = lds128(smem_u32(p));
+    return make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
+}
 
 // RUN: a calibration run of p.n_tokens tokens without outputs; otherwise one decode step.
 // DV > 0 fixes d_v (row addresses become immediate offsets).
@@ -139,6 +149,7 @@ __global__ void __launch_bounds__(32 * kFp32Warps, kFp32Ctas) fp32_tokens_kernel
     };
 
     const int n_tokens = RUN ? p.n_tokens : 1;
+    auto ld4 = [](const float *at) { return staged4<RUN>(at); };
     Unit cur = next_unit();
     if (cur.ok) {
         fetch_state(cur);
@@ -174,9 +185,8 @@ __global__ void __launch_bounds__(32 * kFp32Warps, kFp32Ctas) fp32_tokens_kernel
             }
             for (int u = tid; u < DK; u += nthr) {
                 const int to = (u & 3) * RP + (u >> 2);
-#pragma unroll
-                for (int s = 0; s < NT; ++s) {
-                    if (s >= nt) break;
+#pragma unroll 2
+                for (int s = 0; s < nt; ++s) {
                     const float kv = load_in(rk[s], u, BF16);
                     sk[s][to] = kv;
                     sb[s][to] = rbeta[s] * kv;
@@ -204,10 +214,14 @@ __global__ void __launch_bounds__(32 * kFp32Warps, kFp32Ctas) fp32_tokens_kernel
                 const float alpha = KDA ? 0.f : salpha[s];
                 // S_bar = Lambda S ; r = S_bar^T k
                 float2 rp[2] = {splat2(0.f), splat2(0.f)};
+                float4 kn = ld4(ka), an = KDA ? ld4(aa) : make_float4(alpha, alpha, alpha, alpha);
 #pragma unroll
                 for (int i4 = 0; i4 < RP / 4; ++i4) {
-                    const float4 k4 = *reinterpret_cast<const float4 *>(ka + 4 * i4);
-                    const float4 a4 = KDA ? *reinterpret_cast<const float4 *>(aa + 4 * i4) : make_float4(alpha, alpha, alpha, alpha);
+                    const float4 k4 = kn, a4 = an;
+                    if (i4 + 1 < RP / 4) {
+                        kn = ld4(ka + 4 * i4 + 4);
+                        if (KDA) an = ld4(aa + 4 * i4 + 4);
+                    }
                     const float kk[4] = {k4.x, k4.y, k4.z, k4.w}, av[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
@@ -219,20 +233,24 @@ __global__ void __launch_bounds__(32 * kFp32Warps, kFp32Ctas) fp32_tokens_kernel
                         }
                     }
                 }
+                const float4 v4 = ld4(sv[s] + warp * kG + 4 * cg);
+                float4 bn = ld4(ba), qn = RUN ? bn : ld4(qa);
                 float r[4] = {rp[0].x, rp[0].y, rp[1].x, rp[1].y};
 #pragma unroll
                 for (int m = 8; m <= 16; m <<= 1) {
 #pragma unroll
                     for (int e = 0; e < 4; ++e) r[e] += __shfl_xor_sync(kFull, r[e], m);
                 }
-                const float4 v4 = *reinterpret_cast<const float4 *>(sv[s] + warp * kG + 4 * cg);
                 const float2 d[2] = {make_float2(v4.x - r[0], v4.y - r[1]), make_float2(v4.z - r[2], v4.w - r[3])};
                 // S = S_bar + beta k d^T ; o = S^T q
                 float2 op[2] = {splat2(0.f), splat2(0.f)};
 #pragma unroll
                 for (int i4 = 0; i4 < RP / 4; ++i4) {
-                    const float4 b4 = *reinterpret_cast<const float4 *>(ba + 4 * i4);
-                    const float4 q4 = RUN ? b4 : *reinterpret_cast<const float4 *>(qa + 4 * i4);
+                    const float4 b4 = bn, q4 = qn;
+                    if (i4 + 1 < RP / 4) {
+                        bn = ld4(ba + 4 * i4 + 4);
+                        qn = RUN ? bn : ld4(qa + 4 * i4 + 4);
+                    }
                     const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, qv[4] = {q4.x, q4.y, q4.z, q4.w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
