@@ -217,10 +217,7 @@ __device__ __forceinline__ void tc_pairs(const float (&v)[32], float2 (&y)[16]) 
     for (int i = 0; i < 16; ++i) y[i] = make_float2(v[2 * i], v[2 * i + 1]);
 }
 
-constexpr uint32_t kIdWP = tc_idesc(128, false, true);  // [K; Q] K-major, S_0 MN-major
-constexpr uint32_t kIdG = tc_idesc(64, false, false);   // [K; Q] and K, both K-major
-constexpr uint32_t kIdO = tc_idesc(128, false, false);  // [.; M] and U, both K-major
-constexpr uint32_t kIdS = tc_idesc(128, true, false);   // K^T MN-major, f_C. U K-major
+constexpr uint32_t kIdG = tc_idesc(64, false, false);  // [K; Q] and K (KDA: X and Z), both K-major
 // byte offset of element (row, k) in a K-major bf16 operand of 8-row groups 1024 B apart
 // (64 columns of K: eight 16-byte core matrices per group)
 __device__ __forceinline__ uint32_t tc_k64_off(int row, int k) {
@@ -435,7 +432,7 @@ struct TcUnit {
 // independent).  The fewer, the more of the work that does not depend on the values is repeated,
 // but with few (slot, head) pairs the SMs would be idle: NV = 1 or 2 where all the units then still
 // run at once (KDA, 32 heads: one prompt of 2048 tokens 737 us with NV = 4, 643 with 1; two of 500
-// tokens 190 / 168 with 2).
+// tokens 190 / 168 with 2; GDN, one prompt of 1000: 213 / 192).
 __host__ __device__ constexpr int tc_nv(int64_t pairs, int sms) { return 4 * pairs <= sms ? 1 : 2 * pairs <= sms ? 2 : 4; }
 // The CTA's next unit with work at or after round `round` (left after it); units without work are
 // skipped, their status bits collected.
@@ -470,13 +467,18 @@ __device__ __forceinline__ TcUnit tc_next_unit(const PrefillParams &p, int64_t &
 // the launchers also instantiate no FP8 or row-absmax kernel).  Thread (row, half):
 // row = tensor-memory lane (warps w and w + 4 reach the same lanes), half = 0 / 1 splits
 // a row's value blocks (0-1 / 2-3) or a phase's tasks between the two.
-template <int FMT>
+template <int FMT, int NV>
 __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const PrefillParams p) {
     static_assert(FMT != kFmtS8Row, "the row-absmax format shares a row scale over the value blocks");
     constexpr bool HAD = fmt_had(FMT);
+    constexpr int NC = 32 * NV;  // value columns of a unit
+    constexpr uint32_t kIdWP = tc_idesc(NC, false, true);   // [K; Q] K-major, S_0 MN-major
+    constexpr uint32_t kIdO = tc_idesc(NC, false, false);   // [.; M] and U, both K-major
+    constexpr uint32_t kIdS = tc_idesc(NC, true, false);    // K^T MN-major, f_C. U K-major
     extern __shared__ __align__(128) uint8_t smem[];  // descriptors need 16-byte alignment (no swizzle)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = tid & 127, half = tid >> 7;
+    const int ca = (half * NV + 1) / 2, cb = ((half + 1) * NV + 1) / 2;  // this half's value blocks of the unit
     const uint32_t sb = smem_u32(smem);
     const int T = p.T, Hm = p.Hm;
     const int rec_bytes = p.rec_bytes, rstride = tc_rec_stride(rec_bytes);
@@ -507,8 +509,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
     bool rec_pending = false, mma_pending = false;  // a copy / a product in flight
     int64_t round = 0;
     const bool sorted = p.lengths && p.batch <= kTcMaxSort;
-    auto next_unit = [&]() { return tc_next_unit<4>(p, round, sorted, sb + (uint32_t)kSmOrder, bad_slot, bad_head); };
-    auto rec_of = [&](const TcUnit &n) { return p.state + n.slot * p.slot_bytes + (int64_t)(n.h * 4) * rec_bytes; };
+    auto next_unit = [&]() { return tc_next_unit<NV>(p, round, sorted, sb + (uint32_t)kSmOrder, bad_slot, bad_head); };
+    auto rec_of = [&](const TcUnit &n) { return p.state + n.slot * p.slot_bytes + (int64_t)(n.h * 4 + n.c0) * rec_bytes; };
     // [K; Q] (bf16, natural channel order, K-major), v, g and beta of unit n's piece at p0
     // (cp.async; a masked token is zero, neither decays nor updates)
     auto load_piece = [&](const TcUnit &n, int p0) {
@@ -552,10 +554,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
     auto prefetch = [&](const TcUnit &n) {
         if (tid == 0) {
             fence_proxy_async_smem();
-            mbar_arrive_expect_tx(bar_rec, (uint32_t)(4 * rec_bytes));
+            mbar_arrive_expect_tx(bar_rec, (uint32_t)(NV * rec_bytes));
             uint8_t *const g0 = rec_of(n);
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
+            for (int c = 0; c < NV; ++c)
                 bulk_g2s(sb + (uint32_t)(kSmRec + c * rstride), g0 + (int64_t)c * rec_bytes, (uint32_t)rec_bytes, bar_rec);
         }
         if (tid < 8) cp_async16(s_perm + 16 * tid, p.perm + (int64_t)n.h * 128 + 16 * tid);
@@ -578,7 +580,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
 
         // ---- S_0: record row u = row, reconstructed (FP32, natural scale, transformed domain
         //      with H_32) into tensor-memory lane u; this half's two value blocks ----
-        tc_reconstruct<FMT>(p, sb + (uint32_t)kSmRec, rstride, row, 2 * half, 2 * half + 2, tS);
+        tc_reconstruct<FMT>(p, sb + (uint32_t)kSmRec, rstride, row, ca, cb, tS);
 
 #pragma unroll 1
         for (int p0 = 0; p0 < Tb; p0 += kTcC) {
@@ -593,7 +595,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
             {
                 const int ch = (int)(lds_u8(s_perm + row) & 127u);
 #pragma unroll 1
-                for (int c = 2 * half; c < 2 * half + 2; ++c) {
+                for (int c = ca; c < cb; ++c) {
                     float v[32];
                     tc_ld32(tS + 32 * c, v);
 #pragma unroll
@@ -688,7 +690,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
                     // gamma_t P_t: the output product accumulates onto it
                     const float gt = ldsf(s_gam + 4 * t);
 #pragma unroll 1
-                    for (int c = 0; c < 4; ++c) {
+                    for (int c = 0; c < NV; ++c) {
                         float v[32];
                         tc_ld32(tWP + 32 * c, v);
 #pragma unroll
@@ -729,7 +731,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
                 // gamma_C S_0: the state product accumulates onto it
                 const float gC = ldsf(s_gam + 4 * (kTcC - 1));
 #pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < NV; ++c) {
                     float v[32];
                     tc_ld32(tS + 32 * c, v);
 #pragma unroll
@@ -741,9 +743,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
             if (row < 64) {
                 const int t = row;
                 const float bt = ldsf(s_beta + 4 * t), gt = ldsf(s_gam + 4 * t);
-                const uint32_t vrow = sb + (uint32_t)(kSmV + t * kTcRowV), yrow = sb + (uint32_t)(kSmYU + t * kTcRowY * 4);
+                const uint32_t vrow = sb + (uint32_t)(kSmV + t * kTcRowV + 64 * cur.c0), yrow = sb + (uint32_t)(kSmYU + t * kTcRowY * 4);
 #pragma unroll 1
-                for (int c = 2 * half; c < 2 * half + 2; ++c) {
+                for (int c = ca; c < cb; ++c) {
                     float w[32];
                     tc_ld32(tWP + 32 * c, w);
                     float2 y[16];
@@ -768,23 +770,27 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
             }
             __syncthreads();
             // ---- U = L^-1 Y by forward substitution, in place ----
-            tc_solve<kTcThreads / 32, 4>(sb + (uint32_t)kSmYU, sb + (uint32_t)kSmLP, warp, lane);
+            tc_solve<kTcThreads / 32, NV>(sb + (uint32_t)kSmYU, sb + (uint32_t)kSmLP, warp, lane);
             __syncthreads();
             // ---- U (half 0) and f_C. U (half 1) as three bf16 parts, K-major (value columns n x
             //      tokens s) ----
             {
                 const uint32_t col = sb + (uint32_t)(kSmYU + 4 * row);
                 float uc[64];
+                if (NV == 4 || row < NC) {
 #pragma unroll
-                for (int t = 0; t < 64; ++t) uc[t] = ldsf(col + (uint32_t)(t * kTcRowY * 4));
+                    for (int t = 0; t < 64; ++t) uc[t] = ldsf(col + (uint32_t)(t * kTcRowY * 4));
+                }
                 __syncthreads();  // every column is read: the parts go over L' and Y / U
                 const uint32_t dst = sb + (uint32_t)(half == 0 ? kSmBU : kSmB4);
+                if (NV == 4 || row < NC) {
 #pragma unroll
-                for (int g = 0; g < 8; ++g) {
-                    float x8[8];
+                    for (int g = 0; g < 8; ++g) {
+                        float x8[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) x8[e] = half == 0 ? uc[8 * g + e] : ldsf(s_rev + 4 * (8 * g + e)) * uc[8 * g + e];
-                    split3_store8(dst + tc_k64_off(row, 8 * g), 16384, x8);
+                        for (int e = 0; e < 8; ++e) x8[e] = half == 0 ? uc[8 * g + e] : ldsf(s_rev + 4 * (8 * g + e)) * uc[8 * g + e];
+                        split3_store8(dst + tc_k64_off(row, 8 * g), 16384, x8);
+                    }
                 }
             }
             fence_proxy_async_smem();
@@ -819,9 +825,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
             // ---- o_t = H (gamma_t P_t + (M U)_t) (lanes 64 + t, this half's value blocks) ----
             if (row >= 64) {
                 const int t = row - 64;
-                float *orow = p.o + (((int64_t)b * T + p0 + min(t, nt - 1)) * Hm + mh) * 128;
+                float *orow = p.o + (((int64_t)b * T + p0 + min(t, nt - 1)) * Hm + mh) * 128 + 32 * cur.c0;
 #pragma unroll 1
-                for (int c = 2 * half; c < 2 * half + 2; ++c) {
+                for (int c = ca; c < cb; ++c) {
                     float ov[32];
                     tc_ld32(tWP + 32 * c, ov);
                     float2 y[16];
@@ -840,7 +846,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
         if (timed_out) break;
         // ---- the chunk-final state (tensor-memory lane u = record row u, this half's value
         //      blocks) into the record in place ----
-        tc_requantize<FMT>(p, grec0, row, 2 * half, 2 * half + 2, lane, tS);
+        tc_requantize<FMT>(p, grec0, row, ca, cb, lane, tS);
         cur = nxt;
     }
     // a copy or a product that did not complete in time gets one more bounded wait before

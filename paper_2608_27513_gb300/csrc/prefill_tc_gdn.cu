@@ -8,9 +8,11 @@
 namespace damp {
 
 cudaError_t launch_prefill_tc_gdn(const PrefillParams &p, int fmt, cudaStream_t stream) {
+    const int64_t pairs = (int64_t)p.batch * p.H;
+    const int nv = tc_nv(pairs, sm_count());
     void (*kern)(PrefillParams) = nullptr;
-    if (fmt == kFmtU8H32) kern = prefill_tc_gdn_kernel<kFmtU8H32>;
-    if (fmt == kFmtU8) kern = prefill_tc_gdn_kernel<kFmtU8>;
+    if (fmt == kFmtU8H32) kern = nv == 4 ? prefill_tc_gdn_kernel<kFmtU8H32, 4> : nv == 2 ? prefill_tc_gdn_kernel<kFmtU8H32, 2> : prefill_tc_gdn_kernel<kFmtU8H32, 1>;
+    if (fmt == kFmtU8) kern = nv == 4 ? prefill_tc_gdn_kernel<kFmtU8, 4> : nv == 2 ? prefill_tc_gdn_kernel<kFmtU8, 2> : prefill_tc_gdn_kernel<kFmtU8, 1>;
     if (!kern) return cudaErrorNotSupported;
     const int smem = kTcSmem;
     if (p.rec_bytes > kTcMaxRec || smem > max_smem_per_block()) return cudaErrorNotSupported;
@@ -20,8 +22,7 @@ cudaError_t launch_prefill_tc_gdn(const PrefillParams &p, int fmt, cudaStream_t 
     if (per_sm <= 0 || 2 * smem <= per_sm) return cudaErrorNotSupported;
     cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(kern), smem);
     if (e != cudaSuccess) return e;
-    const int64_t units = (int64_t)p.batch * p.H;
-    const int grid = (int)std::min<int64_t>(units, (int64_t)sm_count());
+    const int grid = (int)std::min<int64_t>(pairs * (4 / nv), (int64_t)sm_count());
     kern<<<grid, kTcThreads, smem, stream>>>(p);
     return cudaGetLastError();
 }

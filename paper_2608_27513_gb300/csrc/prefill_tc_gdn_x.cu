@@ -9,9 +9,11 @@
 namespace damp {
 
 cudaError_t launch_prefill_tc_gdn_x(const PrefillParams &p, int fmt, cudaStream_t stream) {
+    const int64_t pairs = (int64_t)p.batch * p.H;
+    const int nv = tc_nv(pairs, sm_count());
     void (*kern)(PrefillParams) = nullptr;
-    if (fmt == kFmtU4H32) kern = prefill_tc_gdn_kernel<kFmtU4H32>;
-    if (fmt == kFmtU4) kern = prefill_tc_gdn_kernel<kFmtU4>;
+    if (fmt == kFmtU4H32) kern = nv == 4 ? prefill_tc_gdn_kernel<kFmtU4H32, 4> : nv == 2 ? prefill_tc_gdn_kernel<kFmtU4H32, 2> : prefill_tc_gdn_kernel<kFmtU4H32, 1>;
+    if (fmt == kFmtU4) kern = nv == 4 ? prefill_tc_gdn_kernel<kFmtU4, 4> : nv == 2 ? prefill_tc_gdn_kernel<kFmtU4, 2> : prefill_tc_gdn_kernel<kFmtU4, 1>;
     if (!kern) return cudaErrorNotSupported;
     const int smem = kTcSmem;
     if (p.rec_bytes > kTcMaxRec || smem > max_smem_per_block()) return cudaErrorNotSupported;
@@ -21,8 +23,7 @@ cudaError_t launch_prefill_tc_gdn_x(const PrefillParams &p, int fmt, cudaStream_
     if (per_sm <= 0 || 2 * smem <= per_sm) return cudaErrorNotSupported;
     cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(kern), smem);
     if (e != cudaSuccess) return e;
-    const int64_t units = (int64_t)p.batch * p.H;
-    const int grid = (int)std::min<int64_t>(units, (int64_t)sm_count());
+    const int grid = (int)std::min<int64_t>(pairs * (4 / nv), (int64_t)sm_count());
     kern<<<grid, kTcThreads, smem, stream>>>(p);
     return cudaGetLastError();
 }

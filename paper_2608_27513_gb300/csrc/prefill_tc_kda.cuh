@@ -428,12 +428,12 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
             {
                 const uint32_t col = sb + (uint32_t)(kKdYU + 4 * row);
                 float uc[16];
-                if (row < NC) {
+                if (NV == 4 || row < NC) {
 #pragma unroll
                     for (int t = 0; t < 16; ++t) uc[t] = ldsf(col + (uint32_t)((16 * qq + t) * kTcRowY * 4));
                 }
                 __syncthreads();  // every column is read: the parts go over Y / U
-                if (row < NC) {
+                if (NV == 4 || row < NC) {
 #pragma unroll
                     for (int g = 0; g < 2; ++g) split3_store8(sb + tc_k64_off(row, 16 * qq + 8 * g), kd_bu(1), kd_bu(2), uc + 8 * g);
                 }
