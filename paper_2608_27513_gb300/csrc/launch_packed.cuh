@@ -90,6 +90,7 @@ static cudaError_t packed_launch_shape(const StepArgs &a, uint32_t *status, Pack
     out->p = p;
     out->warps = warps;
     // fewer tiles than the grid has warps: still one CTA per SM, the tiles spread evenly over them
+    // (KDA B = 1, 128 tiles: 6.3 us on 128 SMs, 8.3 us on 16 full ones; equal from B = 4)
     out->grid = (int)std::min<int64_t>(std::max<int64_t>(p.total_tiles, 1), (int64_t)sm_count());
     out->smem = p.warp_smem * warps;
     return cudaSuccess;

@@ -109,7 +109,7 @@ static cudaError_t launch_prefill_impl(const StepArgs &a, cudaStream_t stream, u
     } else {
         while (warps > 1 && warps * warp_smem > max_smem_per_block()) --warps;
         if (warps * warp_smem > max_smem_per_block()) return cudaErrorInvalidValue;
-        want = p.total_tiles;
+        want = p.total_tiles;  // few tiles: over all SMs (four tokens of one slot: 16.5 -> 10.4 us)
     }
     p.amax_off = warps * warp_smem;
     const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count());
