@@ -305,6 +305,7 @@ __device__ __forceinline__ void tc_solve(uint32_t yu, uint32_t lt, int warp, int
     };
 #pragma unroll
     for (int i = 0; i < RW; ++i) row(r0 + i, acc[i]);
+    if constexpr (NV < 4) __syncwarp();  // every lane has read Y before a lane of the same columns stores U (warp 0: no barrier between)
     float own[RW][RW];  // L' of this warp's rows among themselves
 #pragma unroll
     for (int a = 0; a < RW - 1; ++a) ltr(r0 + a, own[a]);
