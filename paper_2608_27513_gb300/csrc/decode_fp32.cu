@@ -40,13 +40,15 @@ struct Fp32Params {
     float *o;
     int32_t batch, H, Hqk, dv, V, VG;  // VG: groups of four value blocks per (slot, head)
     int32_t n_tokens;                  // token t's operands lie t * batch rows further on
-    int64_t units;
+    int64_t units;                     // of four value blocks each (pipelined kernel), or tiles
     uint32_t *status;
 };
 
 constexpr int kFp32Warps = 4;
 constexpr int kFp32Ctas = 2;    // CTAs per SM: a third (168 registers a thread) spills, step 47 -> 54 us (below)
 constexpr int kFp32Tokens = 8;  // tokens staged at a time by a calibration run
+constexpr int kFp32TileWarps = 8;
+constexpr int64_t kFp32L2Bytes = 129000000;
 
 // A staged operand vector.  A run's loads keep their place in the program (one group of four rows
 // ahead of their use): left to the compiler, they are all moved to the front of the token, over the
@@ -294,11 +296,108 @@ __global__ void __launch_bounds__(32 * kFp32Warps, kFp32Ctas) fp32_tokens_kernel
     }
 }
 
-template <bool RUN>
-static cudaError_t launch_fp32(const StepArgs &a, int32_t n_tokens, cudaStream_t stream) {
-    Fp32Params p{};
+// The step of the shapes whose CTAs the pipelined kernel cannot fill (launch_fp32_step): one warp
+// per tile of d_k rows x 32 columns, lane j owns column j for all rows, so both sums over the rows
+// are its own (as four chains, in the same order as above: same bits) and every load or store of a
+// row is one 128-byte line.  d_k independent loads in flight per warp, eight warps per SM whatever
+// d_v; bound by HBM latency times what those keep in flight.  Also the single tokens of a
+// calibration run (no outputs: o is null).
+template <int DK, int DV, bool KDA, bool BF16>
+__global__ void __launch_bounds__(32 * kFp32TileWarps, 1) fp32_tile_kernel(const Fp32Params p) {
+    __shared__ __align__(16) float ops[kFp32TileWarps][4][DK];  // k, q, a, beta*k per channel
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int nw = blockDim.x >> 5;
+    float *sk = ops[warp][0];
+    float *sq = ops[warp][1];
+    float *sa = ops[warp][2];
+    float *sb = ops[warp][3];
+
+    const int64_t gw = (int64_t)blockIdx.x * nw + warp;
+    const int64_t nwt = (int64_t)gridDim.x * nw;
+    const int64_t t0 = p.units * gw / nwt;
+    const int64_t t1 = p.units * (gw + 1) / nwt;
+    bool bad_slot = false;
+
+    for (int64_t t = t0; t < t1; ++t) {
+        const int c = (int)(t % p.V);
+        const int64_t bh = t / p.V;
+        const int h = (int)(bh % p.H);
+        const int b = (int)(bh / p.H);
+        if (t == t0 || c == 0) {
+            __syncwarp();
+            const int hq = (h * p.Hqk) / p.H;
+            const int64_t qoff = ((int64_t)b * p.Hqk + hq) * DK;
+            const float beta = p.beta[(int64_t)b * p.H + h];
+            const float alpha = KDA ? 0.f : expf(p.g[(int64_t)b * p.H + h]);
+#pragma unroll
+            for (int u = lane; u < DK; u += 32) {
+                const float kv = load_in(p.k, qoff + u, BF16);
+                sk[u] = kv;
+                sq[u] = load_in(p.q, qoff + u, BF16);
+                sa[u] = KDA ? expf(p.g[((int64_t)b * p.H + h) * DK + u]) : alpha;
+                sb[u] = beta * kv;
+            }
+            __syncwarp();
+        }
+        const int64_t slot = p.slot_idx ? (int64_t)p.slot_idx[b] : (int64_t)b;
+        if (slot < 0 || slot >= p.num_slots) {
+            bad_slot = true;
+            continue;
+        }
+        float *base = p.state + ((slot * p.H + h) * DK) * (int64_t)p.dv + c * kG + lane;
+        // a compile-time row stride (DV > 0) turns every row address into an
+        // immediate offset from one base register
+        const int64_t ld = DV > 0 ? DV : p.dv;
+        float x[DK];
+#pragma unroll
+        for (int u = 0; u < DK; ++u) x[u] = __ldcs(base + u * ld);
+        const float vj = load_in(p.v, ((int64_t)b * p.H + h) * p.dv + c * kG + lane, BF16);
+
+        // S_bar = Lambda S ; r = S_bar^T k
+        float r0 = 0.f, r1 = 0.f, r2 = 0.f, r3 = 0.f;
+#pragma unroll
+        for (int u = 0; u < DK; u += 4) {
+            const float4 a4 = *reinterpret_cast<const float4 *>(sa + u);
+            const float4 k4 = *reinterpret_cast<const float4 *>(sk + u);
+            x[u] *= a4.x;
+            x[u + 1] *= a4.y;
+            x[u + 2] *= a4.z;
+            x[u + 3] *= a4.w;
+            r0 = fmaf(x[u], k4.x, r0);
+            r1 = fmaf(x[u + 1], k4.y, r1);
+            r2 = fmaf(x[u + 2], k4.z, r2);
+            r3 = fmaf(x[u + 3], k4.w, r3);
+        }
+        const float d = vj - ((r0 + r1) + (r2 + r3));
+        // S = S_bar + beta k d^T ; o = S^T q
+        float o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
+#pragma unroll
+        for (int u = 0; u < DK; u += 4) {
+            const float4 b4 = *reinterpret_cast<const float4 *>(sb + u);
+            const float4 q4 = *reinterpret_cast<const float4 *>(sq + u);
+            x[u] = fmaf(b4.x, d, x[u]);
+            x[u + 1] = fmaf(b4.y, d, x[u + 1]);
+            x[u + 2] = fmaf(b4.z, d, x[u + 2]);
+            x[u + 3] = fmaf(b4.w, d, x[u + 3]);
+            o0 = fmaf(x[u], q4.x, o0);
+            o1 = fmaf(x[u + 1], q4.y, o1);
+            o2 = fmaf(x[u + 2], q4.z, o2);
+            o3 = fmaf(x[u + 3], q4.w, o3);
+        }
+        // a fresh copy of the row pointer keeps the compiler from holding all
+        // d_k load addresses live until the stores
+#pragma unroll
+        for (int u = 0; u < DK; ++u) __stcs(base + u * ld, x[u]);
+        if (p.o) p.o[((int64_t)b * p.H + h) * p.dv + c * kG + lane] = (o0 + o1) + (o2 + o3);  // no o: calibration runs
+    }
+    if (bad_slot && lane == 0) atomicOr(p.status, (uint32_t)kDevBadSlot);
+}
+
+
+static cudaError_t fp32_params(const StepArgs &a, Fp32Params &p) {
     static std::atomic<uint32_t *> cache[64];
-    cudaError_t e = symbol_address_cached(&g_status_fp32, cache, &p.status);
+    const cudaError_t e = symbol_address_cached(&g_status_fp32, cache, &p.status);
     if (e != cudaSuccess) return e;
     p.state = static_cast<float *>(a.state);
     p.num_slots = a.num_slots;
@@ -315,23 +414,33 @@ static cudaError_t launch_fp32(const StepArgs &a, int32_t n_tokens, cudaStream_t
     p.dv = a.dv;
     p.V = a.dv / kG;
     p.VG = (p.V + kFp32Warps - 1) / kFp32Warps;
+    return cudaSuccess;
+}
+
+#define DAMP_PICK4(KERN_, DK_, DV_, ...)                                                           \
+    if (a.kda) kern = a.in_bf16 ? KERN_<DK_, DV_, true, true __VA_ARGS__> : KERN_<DK_, DV_, true, false __VA_ARGS__>; \
+    else kern = a.in_bf16 ? KERN_<DK_, DV_, false, true __VA_ARGS__> : KERN_<DK_, DV_, false, false __VA_ARGS__>;
+
+template <bool RUN>
+static cudaError_t launch_fp32(const StepArgs &a, int32_t n_tokens, cudaStream_t stream) {
+    Fp32Params p{};
+    cudaError_t e = fp32_params(a, p);
+    if (e != cudaSuccess) return e;
     p.n_tokens = n_tokens;
     p.units = (int64_t)a.batch * a.H * p.VG;
     if (p.units == 0 || n_tokens == 0) return cudaSuccess;
     void (*kern)(Fp32Params) = nullptr;
-#define DAMP_PICK4(DK_, DV_)                                                                       \
-    if (a.kda) kern = a.in_bf16 ? fp32_tokens_kernel<DK_, DV_, true, true, RUN> : fp32_tokens_kernel<DK_, DV_, true, false, RUN>; \
-    else kern = a.in_bf16 ? fp32_tokens_kernel<DK_, DV_, false, true, RUN> : fp32_tokens_kernel<DK_, DV_, false, false, RUN>;
+#define DAMP_COMMA_RUN , RUN
 #define DAMP_PICK(DK_)                                                                             \
     if (a.dk == DK_) {                                                                             \
-        if (a.dv == 128) { DAMP_PICK4(DK_, 128) }                                                  \
-        else { DAMP_PICK4(DK_, 0) }                                                                \
+        if (a.dv == 128) { DAMP_PICK4(fp32_tokens_kernel, DK_, 128, DAMP_COMMA_RUN) }              \
+        else { DAMP_PICK4(fp32_tokens_kernel, DK_, 0, DAMP_COMMA_RUN) }                            \
     }
-    DAMP_PICK(32)
+    if constexpr (RUN) { DAMP_PICK(32) }  // (a step of d_k = 32 never comes here)
     DAMP_PICK(64)
     DAMP_PICK(128)
 #undef DAMP_PICK
-#undef DAMP_PICK4
+#undef DAMP_COMMA_RUN
     if (!kern) return cudaErrorInvalidValue;
     const int warps = std::min(p.V, kFp32Warps), smem = a.dk * warps * kG * 4;
     if ((e = ensure_smem_limit(reinterpret_cast<const void *>(kern), smem)) != cudaSuccess) return e;
@@ -340,7 +449,51 @@ static cudaError_t launch_fp32(const StepArgs &a, int32_t n_tokens, cudaStream_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_fp32_step(const StepArgs &a, cudaStream_t stream) { return launch_fp32<false>(a, 1, stream); }
+static cudaError_t launch_fp32_tile(const StepArgs &a, cudaStream_t stream) {
+    Fp32Params p{};
+    const cudaError_t e = fp32_params(a, p);
+    if (e != cudaSuccess) return e;
+    p.n_tokens = 1;
+    p.units = (int64_t)a.batch * a.H * p.V;  // tiles
+    if (p.units == 0) return cudaSuccess;
+    void (*kern)(Fp32Params) = nullptr;
+#define DAMP_PICK(DK_)                                                                             \
+    if (a.dk == DK_) {                                                                             \
+        if (a.dv == 64) { DAMP_PICK4(fp32_tile_kernel, DK_, 64) }                                  \
+        else if (a.dv == 128) { DAMP_PICK4(fp32_tile_kernel, DK_, 128) }                           \
+        else { DAMP_PICK4(fp32_tile_kernel, DK_, 0) }                                              \
+    }
+    DAMP_PICK(32)
+    DAMP_PICK(64)
+    DAMP_PICK(128)
+#undef DAMP_PICK
+    if (!kern) return cudaErrorInvalidValue;
+    const int64_t want = (p.units + kFp32TileWarps - 1) / kFp32TileWarps;
+    kern<<<(int)std::min<int64_t>(want, (int64_t)sm_count()), 32 * kFp32TileWarps, 0, stream>>>(p);
+    return cudaGetLastError();
+}
+#undef DAMP_PICK4
+
+// The pipelined kernel where its CTAs are full: two CTAs of up to four warps per SM move a 32 KB
+// (64 x 128) to 64 KB state each, so it needs tall tiles and whole groups of four value blocks
+// (or one of three).  Measured, pipelined / tile kernel, H = 32, states from memory:
+//   d_k = 128: d_v = 96, B = 64: 38 / 57 us; 128: 45 / 48; 256: 117 / 145; 1024: 488 / 578;
+//     a group with idle warps: d_v = 32: 23 / 20, 64: 29 / 27, 160: 116 / 90, 288: 165 / 163;
+//   d_k = 64: d_v = 128, B = 256: 84 / 98, but from L2 (B = 64) 17 / 15; 64, B = 256: 55 / 52; 160: 214 / 131;
+//   d_k = 32: 32 x 32, B = 256: 40 / 17; 32 x 128: even, from L2 13 / 9.
+// A call of few units gives each its own CTA, where the tile kernel packs eight tiles into one:
+//   128 x 32, B = 8: 5 / 11; 64 x 64, B = 8: 3.6 / 4.3; 128 x 160, B = 2: 9.3 / 11.
+static bool fp32_pipelined(const StepArgs &a) {
+    const int64_t V = a.dv / kG, VG = (V + kFp32Warps - 1) / kFp32Warps, units = (int64_t)a.batch * a.H * VG;
+    const bool full = V % kFp32Warps == 0 || V == 3;
+    if (a.dk == 128 && (full || units <= sm_count())) return true;
+    if (a.dk < 64 || VG > 1) return false;
+    return units <= 2 * sm_count() || (full && (int64_t)a.batch * a.H * a.dk * a.dv * 4 > kFp32L2Bytes);
+}
+
+cudaError_t launch_fp32_step(const StepArgs &a, cudaStream_t stream) {
+    return fp32_pipelined(a) ? launch_fp32<false>(a, 1, stream) : launch_fp32_tile(a, stream);
+}
 cudaError_t launch_fp32_run(const StepArgs &a, int32_t n_tokens, cudaStream_t stream) {
     return launch_fp32<true>(a, n_tokens, stream);
 }
