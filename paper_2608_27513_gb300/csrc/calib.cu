@@ -153,13 +153,26 @@ __global__ void __launch_bounds__(32 * kEeWarps) calib_error_energy_kernel(const
     }
 }
 
-// One warp per 32 accumulators: lane u of warp (head, 32 channels) for KDA, lane i of a warp
-// of 32 held heads for GDN (a head's sum counts for all its channels).  Every lane adds its
-// rows one after the other (a fixed order); the rows stream in by 4-byte cp.async (g is
-// 4-byte aligned) through a ring of kLdStages x kLdRows rows, each lane reading only what it
-// copied, so that a warp keeps 56 KB in flight: with H = 32 heads only 128 warps run (KDA,
-// 32 documents x 256 tokens, 134 MB: 12.6 us in L2's wake; plain loads, a few in flight per
-// lane, took about 0.9 ms).
+// Few rows: a thread per accumulator adds its rows straight from memory.
+__global__ void calib_log_decay_few_kernel(const float *g, int32_t batch, int32_t H, int32_t Hm, const int32_t *head_map,
+                                           int32_t dk, int32_t kda, float *G_acc) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)H * dk) return;
+    const int h = (int)(i / dk), u = (int)(i % dk);
+    const int m = calib_model_head(head_map, h, Hm);
+    if (m < 0) return;
+    float s = 0.f;
+    for (int b = 0; b < batch; ++b) s += kda ? g[((int64_t)b * Hm + m) * dk + u] : g[(int64_t)b * Hm + m];
+    G_acc[(int64_t)m * dk + u] += s;
+}
+
+// Many rows: one warp per 32 accumulators, lane u of warp (head, 32 channels) for KDA, lane i of a
+// warp of 32 held heads for GDN (a head's sum counts for all its channels).  Every lane adds its
+// rows one after the other (a fixed order, the same as above); the rows stream in by 4-byte
+// cp.async (g is 4-byte aligned) through a ring of kLdStages x kLdRows rows, each lane reading only
+// what it copied, so that a warp keeps 56 KB in flight: with H = 32 heads only 128 warps run (KDA).
+// Bound by the chain of a lane's adds (about 17 cycles a row).  KDA, 32 documents x 256 tokens (8192
+// rows, 134 MB): 73 us, 1120 us with a thread per accumulator; GDN 83 and 114 us.
 constexpr int kLdRows = 64, kLdStages = 8;
 constexpr int kLdSmem = kLdStages * kLdRows * 32 * 4;
 
@@ -296,6 +309,15 @@ cudaError_t launch_calib_error_energy(const float *S, int32_t batch, int32_t H, 
 
 cudaError_t launch_calib_log_decay(const float *g, int32_t batch, int32_t H, int32_t Hm, const int32_t *head_map,
                                    int32_t dk, int32_t kda, float *G_acc, cudaStream_t stream) {
+    // The ring's start and, for GDN, a warp's 32 rows of G_acc cost more than few rows take, ring /
+    // thread per accumulator: KDA 1 row 2.3 / 1.9 us, 12 rows 2.4 / 2.4, 64 rows 2.6 / 4.5; GDN 1 row
+    // 10.4 / 1.8, 256 rows 12.6 / 5.2, 1500 rows 24.0 / 22.9, 2048 rows 28.6 / 30.1 (32 heads, d_k 128).
+    if (batch < (kda ? 12 : 1792)) {
+        const int64_t n = (int64_t)H * dk;
+        calib_log_decay_few_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(g, batch, H, Hm, head_map, dk, kda,
+                                                                                      G_acc);
+        return cudaGetLastError();
+    }
     const int64_t grid = kda ? (int64_t)H * (dk / 32) : (H + 31) / 32;
     const auto kern = kda ? calib_log_decay_kernel<true> : calib_log_decay_kernel<false>;
     const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(kern), kLdSmem);

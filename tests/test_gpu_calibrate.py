@@ -10,6 +10,7 @@ import workloads as wl
 from oracle import calibrate, core, runs
 from paper_2608_27513_gb300 import calibration
 from tests import parity as P
+from tests.timing import assert_at_most
 
 pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda:0")
@@ -175,3 +176,27 @@ def test_log_decay_sums_in_row_order(rows, kda):
     G = damp.calib_log_decay(L, P.to_dev(g, DEV), torch.zeros((H, dk), device=DEV)).cpu().numpy()
     ref = np.add.accumulate(g, axis=0, dtype=np.float32)[-1]
     assert np.array_equal(G, ref if kda else np.repeat(ref[:, None], dk, axis=1))
+
+
+@pytest.mark.parametrize("kda,rows", [(True, 11), (True, 12), (True, 13), (False, 1791), (False, 1792), (False, 1800),
+                                      (False, 2111)])
+def test_log_decay_sums_on_both_sides_of_the_line(kda, rows):
+    """Few rows (a thread per accumulator) and many (the ring) add in the same order."""
+    H, dk = 35 if not kda else 3, 64
+    L = damp.Layout(H, H, dk, 64, 0, 0)
+    rng = np.random.default_rng(rows)
+    g = (-np.exp(rng.uniform(-6, 0, (rows, H, dk) if kda else (rows, H)))).astype(np.float32)
+    G = damp.calib_log_decay(L, P.to_dev(g, DEV), torch.zeros((H, dk), device=DEV)).cpu().numpy()
+    ref = np.add.accumulate(g, axis=0, dtype=np.float32)[-1]
+    assert np.array_equal(G, ref if kda else np.repeat(ref[:, None], dk, axis=1))
+
+
+@pytest.mark.parametrize("rows", [1, 256])
+def test_few_rows_of_scalar_gates_take_no_longer_than_of_channel_gates(rows):
+    """GDN's log-decay sums read d_k times less than KDA's: at most twice the time (three to five
+    times where one warp writes 32 heads' accumulators after few rows)."""
+    H, dk = 32, 128
+    L = damp.Layout(H, H, dk, 128, 0, 0)
+    G = torch.zeros((H, dk), device=DEV)
+    gdn, kda = -torch.rand(rows, H, device=DEV), -torch.rand(rows, H, dk, device=DEV)
+    assert_at_most(lambda: damp.calib_log_decay(L, gdn, G), lambda: damp.calib_log_decay(L, kda, G), 2.0, f"{rows} rows")
