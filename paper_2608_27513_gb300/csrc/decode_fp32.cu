@@ -494,8 +494,32 @@ static bool fp32_pipelined(const StepArgs &a) {
 cudaError_t launch_fp32_step(const StepArgs &a, cudaStream_t stream) {
     return fp32_pipelined(a) ? launch_fp32<false>(a, 1, stream) : launch_fp32_tile(a, stream);
 }
+// A run of a few tokens has too little to gain from the states staying in registers: single steps
+// on the tile kernel.  Per 12 tokens of 32 documents with the samples' error passes, run / steps:
+// one token a run: GDN 128 x 128 398 / 359 us, 64 x 64 222 / 174, 32 x 32 158 / 102, KDA 128 x 64 256
+// / 223, but KDA 128 x 128 366 / 386; two: GDN 128 x 128 212 / 282, 64 x 64 119 / 125, 32 x 32 86 /
+// 73; three: GDN 32 x 32 even; four: GDN 32 x 32 51 / 58, 32 x 128 78 / 119.
+static bool fp32_run_pays(const StepArgs &a, int32_t n_tokens) {
+    const int64_t V = a.dv / kG, rows = (int64_t)n_tokens * a.dk;
+    if (n_tokens == 1) return a.kda && a.dk == 128 && (V % kFp32Warps == 0 || V == 3);
+    return rows >= 128;
+}
+
 cudaError_t launch_fp32_run(const StepArgs &a, int32_t n_tokens, cudaStream_t stream) {
-    return launch_fp32<true>(a, n_tokens, stream);
+    if (fp32_run_pays(a, n_tokens)) return launch_fp32<true>(a, n_tokens, stream);
+    const int64_t B = a.batch, esz = a.in_bf16 ? 2 : 4;
+    const int64_t sq = B * a.Hqk * a.dk * esz, sv = B * a.H * a.dv * esz, sg = B * a.H * (a.kda ? a.dk : 1);
+    StepArgs t = a;
+    for (int32_t i = 0; i < n_tokens; ++i) {
+        t.q = static_cast<const uint8_t *>(a.q) + i * sq;
+        t.k = static_cast<const uint8_t *>(a.k) + i * sq;
+        t.v = static_cast<const uint8_t *>(a.v) + i * sv;
+        t.g = a.g + i * sg;
+        t.beta = a.beta + i * B * a.H;
+        const cudaError_t e = launch_fp32_tile(t, stream);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t take_status_fp32(uint32_t *bits) {

@@ -89,3 +89,52 @@ def test_narrow_states_keep_pace_with_square_ones(dk, dv, batch, square_batch):
         return lambda: damp.fp32_gdn_decode_step(L, S, d["q"], d["k"], d["v"], d["g"], d["beta"], o=o)
     assert batch * dk * dv == square_batch * 128 * 128
     assert_at_most(call(dk, dv, batch), call(128, 128, square_batch), 2.0, f"{dk} x {dv}")
+
+
+@pytest.mark.parametrize("kind,dk,dv,T,every", [("kda", 128, 128, 21, 8), ("gdn", 128, 160, 17, 8), ("gdn", 64, 96, 7, 2),
+                                                ("kda", 64, 256, 9, 4), ("gdn", 32, 64, 11, 5), ("kda", 32, 32, 5, 1)])
+def test_documents_of_a_calibration_run_equal_their_own_run(kind, dk, dv, T, every):
+    """A run over 12 documents (384 units and more: several per CTA, each over all tokens between two
+    samples, and single steps where a run is short) leaves every document the states that a run of
+    its own gives it, bit for bit."""
+    docs = 12
+    w = _workload(kind, dk, dv, docs)
+    L = damp.Layout(w.heads, w.qk_heads, dk, dv, 0, 0)
+    inputs = wl.torch_step_inputs(w, T, DEV)
+    st = {n: torch.stack([d[n] for d in inputs]) for n in ("q", "k", "v", "g", "beta")}
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(53)
+    S = 0.3 * torch.randn(docs, w.heads, dk, dv, generator=gen, device=DEV)
+    alone = S.clone()
+
+    def run(s, sl):
+        E, G = (torch.zeros((w.heads, dk), device=DEV) for _ in range(2))
+        damp.calib_accumulate(L, kind, s, *(st[n][:, sl].contiguous() for n in ("q", "k", "v", "g", "beta")), E, G, every)
+    run(S, slice(0, docs))
+    for b in range(docs):
+        run(alone[b:b + 1], slice(b, b + 1))
+    assert torch.equal(S, alone)
+
+
+@pytest.mark.parametrize("dk,dv", [(32, 32), (64, 64)])
+def test_a_sample_every_token_costs_no_more_than_single_steps(dk, dv):
+    """calib_accumulate with every = 1 takes at most 1.2 times its steps and error passes called one
+    by one (which write outputs as well); 1.3 to 1.6 times where one token starts a whole run."""
+    docs, T = 32, 12
+    w = _workload("gdn", dk, dv, docs, qk_heads=32)
+    L = damp.Layout(w.heads, w.qk_heads, dk, dv, 0, 0)
+    inputs = wl.torch_step_inputs(w, T, DEV)
+    st = {n: torch.stack([d[n] for d in inputs]) for n in ("q", "k", "v", "g", "beta")}
+    S = damp.new_fp32_state(L, docs, DEV)
+    o = torch.empty(docs, w.heads, dv, device=DEV)
+    E, G = (torch.zeros((w.heads, dk), device=DEV) for _ in range(2))
+
+    def single():
+        for d in inputs:
+            damp.fp32_gdn_decode_step(L, S, d["q"], d["k"], d["v"], d["g"], d["beta"], o=o)
+            damp.calib_error_energy(L, S, E)
+        damp.calib_log_decay(L, st["g"].flatten(0, 1), G)
+
+    def one_call():
+        damp.calib_accumulate(L, "gdn", S, st["q"], st["k"], st["v"], st["g"], st["beta"], E, G, 1)
+    assert_at_most(one_call, single, 1.2, f"{dk} x {dv}")
