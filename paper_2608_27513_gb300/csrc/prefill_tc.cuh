@@ -60,7 +60,7 @@ constexpr int kSmScal = 181248; // a, beta, gamma, f_C. (64 floats each), pi, g,
 constexpr int kTcRowL = 68;     // floats per row of L'^T
 constexpr int kTcRowY = 132;    // floats per row of Y / U
 constexpr int kTcRowV = 272;    // bytes per row of v
-constexpr int kTcMaxSort = 512;  // batch rows up to which a ragged chunk's units are ordered by length
+constexpr int kTcMaxSort = 256;  // batch rows up to which a ragged chunk's units are ordered by length
 constexpr int kSmOrder = kSmScal + 1472;
 constexpr int kTcSmem = kSmOrder + 2 * kTcMaxSort;
 constexpr int kTcMaxRec = 8192; // largest record (d_k = 128): four fit in [kSmRec, kSmV)
@@ -412,13 +412,24 @@ __device__ __forceinline__ void tc_requantize(const PrefillParams &p, uint8_t *g
 // (up to kTcMaxSort rows: `order`, uint16 in shared memory, filled by tc_sort_rows), so that the
 // CTAs with the longest units get the shortest ones next.  KDA, 13 rows of up to 133 tokens x 32
 // heads (416 units on 152 SMs): 176 us in batch order, 134 us so.
-__device__ __forceinline__ void tc_sort_rows(const PrefillParams &p, uint32_t order) {
+// The order's cost grows with the square of the rows, in every CTA: 1.7 us for 256 rows (from shared
+// memory, one comparison per pair; 3.4 us before), 15 us for 512 from global memory (GDN, 512 rows of
+// 64 tokens x 2 heads: 114.5 us in batch order, 129 us so), where each CTA has enough units that
+// their order matters little.
+__device__ __forceinline__ void tc_sort_rows(const PrefillParams &p, uint32_t order, uint32_t scratch) {
+    // (length, up to 2^22; the earlier of equal rows) as one number, larger first and distinct
+    static_assert(kTcMaxSort <= 512, "a row's number takes nine bits of its key");
+    const int n4 = (p.batch + 3) & ~3;
+    for (int b = threadIdx.x; b < n4; b += blockDim.x)  // keys past the batch: 0, below every row's
+        sts32(scratch + 4 * b, b < p.batch ? (uint32_t)min(min(max(p.lengths[b], 0), p.T), (1 << 22) - 1) * 512u + 512u - (uint32_t)b : 0u);
+    __syncthreads();
     for (int b = threadIdx.x; b < p.batch; b += blockDim.x) {
-        const int len = p.lengths[b];
+        const uint32_t key = lds32(scratch + 4 * b);
         int rank = 0;
-        for (int c = 0; c < p.batch; ++c) {
-            const int other = p.lengths[c];
-            rank += other > len || (other == len && c < b);
+#pragma unroll 4
+        for (int c = 0; c < n4; c += 4) {
+            const uint4 w = lds128(scratch + 4 * c);
+            rank += (w.x > key) + (w.y > key) + (w.z > key) + (w.w > key);
         }
         asm volatile("st.shared.u16 [%0], %1;" ::"r"(order + 2 * rank), "h"((unsigned short)b) : "memory");
     }
@@ -497,7 +508,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const Pre
         mbar_init(bar_mma, 1);
         fence_mbar_init();
     }
-    if (p.lengths && p.batch <= kTcMaxSort) tc_sort_rows(p, sb + (uint32_t)kSmOrder);
+    if (p.lengths && p.batch <= kTcMaxSort) tc_sort_rows(p, sb + (uint32_t)kSmOrder, sb + (uint32_t)kSmB1);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

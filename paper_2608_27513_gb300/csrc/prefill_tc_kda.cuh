@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const Pre
         mbar_init(bar_mma, 1);
         fence_mbar_init();
     }
-    if (p.lengths && p.batch <= kTcMaxSort) tc_sort_rows(p, sb + (uint32_t)kKdOrder);
+    if (p.lengths && p.batch <= kTcMaxSort) tc_sort_rows(p, sb + (uint32_t)kKdOrder, sb + (uint32_t)kKdZ);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
