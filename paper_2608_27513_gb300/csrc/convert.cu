@@ -19,7 +19,7 @@
 // next item's codes while the current one is computed.  B = 64, H = 32, d = 128, K_hi = 16 (134
 // MB FP32 + 41 MB packed): quantize 35.8 us, 4.9 TB/s (B = 256: 128 us, 5.5 TB/s), against 54.8
 // and 169 us with a row per lane from memory; dequantize 38 us against 74 us.  HBM-bound.
-// pack and unpack: one warp per record, lane l owns packed rows l, l + 32, ...
+// pack and unpack, and dequantize at d_k = 32: one warp per record, lane l owns packed rows l, l + 32, ...
 #include "damp_common.cuh"
 #include "damp_internal.h"
 #include "formats.cuh"
@@ -47,7 +47,7 @@ struct ConvParams {
     uint32_t *status;
 };
 
-enum ConvOp { kPackTiers = 2, kUnpackTiers = 3 };
+enum ConvOp { kDequantize = 1, kPackTiers = 2, kUnpackTiers = 3 };
 
 // (batch row, head, value block, row group) of an item, and whether its slot and head are valid
 struct ConvItem {
@@ -276,15 +276,18 @@ __global__ void __launch_bounds__(32 * kCvWarps) dequantize_kernel(const ConvPar
     w.report(lane);
 }
 
+// pack and unpack, and dequantize at d_k = 32: a record is a single item there, without a next one
+// for a warp's loads to run ahead to, and the tile only adds its way through shared memory.
 template <int R, int FMT, int OP>
 __global__ void __launch_bounds__(256) tiers_kernel(const ConvParams p) {
-    constexpr int CB = fmt_u4(FMT) ? 16 : 32;  // code bytes per row and value block
+    constexpr bool HAD = fmt_had(FMT), U4 = fmt_u4(FMT);
+    constexpr int CB = U4 ? 16 : 32;  // code bytes per row and value block
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwt = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int K = p.K;
     const int lo = p.dk - K;
-    bool bad_slot = false;
+    bool bad_slot = false, bad_head = false;
     for (int64_t t = gw; t < p.total_tiles; t += nwt) {
         const int c = (int)(t % p.V);
         const int64_t bh = t / p.V;
@@ -295,6 +298,11 @@ __global__ void __launch_bounds__(256) tiers_kernel(const ConvParams p) {
             bad_slot = true;
             continue;
         }
+        const int mh = OP == kDequantize && p.head_map ? p.head_map[h] : h;  // row of S
+        if (OP == kDequantize && (mh < 0 || mh >= p.Hm)) {
+            bad_head = true;
+            continue;
+        }
         uint8_t *rec = p.state + slot * p.slot_bytes + (int64_t)(h * p.V + c) * p.rec_bytes;
 #pragma unroll
         for (int i = 0; i < R; ++i) {
@@ -302,34 +310,62 @@ __global__ void __launch_bounds__(256) tiers_kernel(const ConvParams p) {
             if (u < K) continue;  // FP16 rows: column-mapped loop below
             const int r = u - K;
             uint32_t *mrec = reinterpret_cast<uint32_t *>(rec + p.meta_off + 4 * r);
-            // logical tiers <-> record, 32-bit words
-            const int64_t row_bytes = (int64_t)p.V * CB;
-            uint32_t *crow = reinterpret_cast<uint32_t *>(p.codes + ((((int64_t)b * p.H + h) * lo + r) * row_bytes + c * CB));
-            uint32_t *mrow = reinterpret_cast<uint32_t *>(p.meta) + (((int64_t)b * p.H + h) * lo + r) * p.V + c;
-#pragma unroll
-            for (int m = 0; m < CB / 16; ++m) {
-                uint32_t *r4 = reinterpret_cast<uint32_t *>(rec + p.codes_off + lo_chunk_off(r, m, lo));
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (OP == kPackTiers) r4[e] = crow[4 * m + e];
-                    else crow[4 * m + e] = r4[e];
+            if (OP == kDequantize) {
+                const int n = p.perm[(int64_t)h * p.dk + u] & (p.dk - 1);  // d_k is a power of two
+                float *row = p.S + ((((int64_t)b * p.Hm + mh) * p.dk + n) * p.dv + c * kG);
+                float2 x[16];
+                const uint4 c0 = *reinterpret_cast<const uint4 *>(rec + p.codes_off + lo_chunk_off(r, 0, lo));
+                if (U4) {
+                    const uint32_t w[4] = {c0.x, c0.y, c0.z, c0.w};
+                    dequantize_group_u4(w, *mrec, 1.0f, x);
+                } else {
+                    const uint4 c1 = *reinterpret_cast<const uint4 *>(rec + p.codes_off + lo_chunk_off(r, 1, lo));
+                    const uint32_t w[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+                    if (FMT == kFmtE4M3) dequantize_group_e4m3(w, __uint_as_float(*mrec), 1.0f, x);
+                    else dequantize_group(w, *mrec, 1.0f, x);
                 }
+                if (HAD) hadamard_pairs(x);
+#pragma unroll
+                for (int m = 0; m < 8; ++m)
+                    reinterpret_cast<float4 *>(row)[m] = make_float4(x[2 * m].x, x[2 * m].y, x[2 * m + 1].x, x[2 * m + 1].y);
+            } else {
+                // logical tiers <-> record, 32-bit words
+                const int64_t row_bytes = (int64_t)p.V * CB;
+                uint32_t *crow = reinterpret_cast<uint32_t *>(p.codes + ((((int64_t)b * p.H + h) * lo + r) * row_bytes + c * CB));
+                uint32_t *mrow = reinterpret_cast<uint32_t *>(p.meta) + (((int64_t)b * p.H + h) * lo + r) * p.V + c;
+#pragma unroll
+                for (int m = 0; m < CB / 16; ++m) {
+                    uint32_t *r4 = reinterpret_cast<uint32_t *>(rec + p.codes_off + lo_chunk_off(r, m, lo));
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (OP == kPackTiers) r4[e] = crow[4 * m + e];
+                        else crow[4 * m + e] = r4[e];
+                    }
+                }
+                if (OP == kPackTiers) *mrec = *mrow;
+                else *mrow = *mrec;
             }
-            if (OP == kPackTiers) *mrec = *mrow;
-            else *mrow = *mrec;
         }
         // ---- FP16 rows, lane = column, two rows per 32-bit word ----
         for (int u = 0; u < K; u += 2) {
             const bool two = u + 1 < K;
             uint32_t *word = reinterpret_cast<uint32_t *>(rec + hi_elem_off(u, lane));
-            uint16_t *t0 = p.hi + ((((int64_t)b * p.H + h) * K + u) * p.dv + c * kG + lane);
-            uint16_t *t1 = two ? t0 + p.dv : nullptr;
-            if (OP == kPackTiers) {
-                *word = (uint32_t)*t0 | ((uint32_t)(two ? *t1 : 0) << 16);
+            if (OP == kDequantize) {
+                float *r0 = p.S + ((((int64_t)b * p.Hm + mh) * p.dk + (p.perm[(int64_t)h * p.dk + u] & (p.dk - 1))) * p.dv + c * kG + lane);
+                float *r1 = two ? p.S + ((((int64_t)b * p.Hm + mh) * p.dk + (p.perm[(int64_t)h * p.dk + u + 1] & (p.dk - 1))) * p.dv + c * kG + lane) : nullptr;
+                const float2 f = h2_to_f2(*word);
+                *r0 = f.x;
+                if (two) *r1 = f.y;
             } else {
-                const uint32_t w = *word;
-                *t0 = (uint16_t)(w & 0xffffu);
-                if (two) *t1 = (uint16_t)(w >> 16);
+                uint16_t *t0 = p.hi + ((((int64_t)b * p.H + h) * K + u) * p.dv + c * kG + lane);
+                uint16_t *t1 = two ? t0 + p.dv : nullptr;
+                if (OP == kPackTiers) {
+                    *word = (uint32_t)*t0 | ((uint32_t)(two ? *t1 : 0) << 16);
+                } else {
+                    const uint32_t w = *word;
+                    *t0 = (uint16_t)(w & 0xffffu);
+                    if (two) *t1 = (uint16_t)(w >> 16);
+                }
             }
         }
         // zero the record padding so packed pools compare bit for bit
@@ -338,7 +374,8 @@ __global__ void __launch_bounds__(256) tiers_kernel(const ConvParams p) {
             if (lane < p.rec_bytes - used) rec[used + lane] = 0;
         }
     }
-    if (lane == 0 && bad_slot) atomicOr(p.status, (uint32_t)kDevBadSlot);
+    if (lane == 0 && (bad_slot || bad_head))
+        atomicOr(p.status, (bad_slot ? (uint32_t)kDevBadSlot : 0u) | (bad_head ? (uint32_t)kDevBadHead : 0u));
 }
 
 static cudaError_t conv_params(const ConvArgs &a, ConvParams &p) {
@@ -393,8 +430,10 @@ static cudaError_t launch_tiers(const ConvArgs &a, cudaStream_t stream) {
 #define DAMP_TIERS2(F_) tiers_kernel<2, F_, OP>
 #define DAMP_TIERS4(F_) tiers_kernel<4, F_, OP>
     if (a.dk == 32) DAMP_PICK_FMT(DAMP_TIERS1)
-    if (a.dk == 64) DAMP_PICK_FMT(DAMP_TIERS2)
-    if (a.dk == 128) DAMP_PICK_FMT(DAMP_TIERS4)
+    if constexpr (OP != kDequantize) {
+        if (a.dk == 64) DAMP_PICK_FMT(DAMP_TIERS2)
+        if (a.dk == 128) DAMP_PICK_FMT(DAMP_TIERS4)
+    }
     if (!kern) return cudaErrorInvalidValue;
     kern<<<grid, 32 * warps, 0, stream>>>(p);
     return cudaGetLastError();
@@ -423,7 +462,12 @@ static cudaError_t launch_convert(const ConvArgs &a, cudaStream_t stream) {
 }
 
 cudaError_t launch_quantize(const ConvArgs &a, cudaStream_t s) { return launch_convert<true>(a, s); }
-cudaError_t launch_dequantize(const ConvArgs &a, cudaStream_t s) { return launch_convert<false>(a, s); }
+// d_k = 32, rows straight to S / through the tiles: d_v = 64, H = 32, B = 256 UINT8 25.3 / 29.6 us,
+// UINT4 23.6 / 29.9; d_v = 256, B = 1024 421 / 430; one request of 32 x 32 4.2 / 4.6.  From d_k = 64
+// the tiles win: 64 x 32, B = 256 24.6 / 20.9.
+cudaError_t launch_dequantize(const ConvArgs &a, cudaStream_t s) {
+    return a.dk == 32 ? launch_tiers<kDequantize>(a, s) : launch_convert<false>(a, s);
+}
 cudaError_t launch_pack_tiers(const ConvArgs &a, cudaStream_t s) { return launch_tiers<kPackTiers>(a, s); }
 cudaError_t launch_unpack_tiers(const ConvArgs &a, cudaStream_t s) { return launch_tiers<kUnpackTiers>(a, s); }
 

@@ -142,3 +142,28 @@ def test_conversions_of_a_batch_equal_those_of_single_rows(fmt, dk, dv, K):
         assert torch.equal(back[b:b + 1], damp.dequantize_state(L, pool, perm, batch=1, slot_idx=idx[b:b + 1].clone()))
     hi = perm[:, :K].long()[None, :, :, None].expand(len(rows), H, K, dv)
     assert torch.equal(torch.gather(back[rows], 2, hi), torch.gather(S[rows].half().float(), 2, hi))
+
+
+@pytest.mark.parametrize("fmt", [core.FMT_U8_H32, core.FMT_U8, *NEW])
+@pytest.mark.parametrize("K", [0, 7, 32])
+def test_dequantize_of_32_channels_matches_oracle(fmt, K):
+    """d_k = 32 has a kernel of its own (a record per warp): K_hi at both ends and odd, three value
+    blocks, more records than the grid has warps, scattered slots and one outside the pool."""
+    B, H, dk, dv, n = 1100, 3, 32, 96, 1103
+    w = wl.Workload("t", "kda", B, H, H, dk, dv, K, 1, 1, "fp32", 7, fmt)
+    S = wl.random_states(63, B * H, dk, dv)
+    perms = np.stack([np.random.default_rng(h).permutation(dk) for h in range(H)]).astype(np.uint8)
+    perm_units = np.tile(perms, (B, 1))
+    tiers = core.pack_heads(perm_units, S, K, fmt)
+    want = core.unpack_heads(perm_units, *tiers, K, fmt, dk, dv).reshape(B, H, dk, dv)
+    L = P.layout_of(w)
+    pool = damp.new_state(L, n, DEV)
+    idx = torch.from_numpy(np.random.default_rng(64).permutation(n)[:B].astype(np.int32)).to(DEV)
+    damp.pack_tiers(L, *P.tiers_to_dev(w, tiers, B, DEV), pool, slot_idx=idx)
+    idx[500] = n
+    got = damp.dequantize_state(L, pool, P.to_dev(perms, DEV), batch=B, slot_idx=idx).cpu().numpy()
+    assert damp.device_status() == damp.DEV_BAD_SLOT
+    assert not got[500].any()
+    want[500] = 0
+    scale = np.abs(want).max(axis=-1, keepdims=True) + 1e-30
+    assert np.all(np.abs(got - want) <= 1e-6 * scale)
