@@ -20,6 +20,7 @@ from __future__ import annotations
 import ctypes
 import functools
 from dataclasses import dataclass, field
+from numbers import Integral
 
 from ._lib import DampLayout, DampLibraryError, lib
 
@@ -70,6 +71,8 @@ class Layout:
     head_map: object = field(default=None, compare=False, repr=False)
 
     def __post_init__(self):
+        sizes = (self.num_heads, self.num_qk_heads, self.d_k, self.d_v, self.k_hi, self.lo_format, self.model_heads)
+        object.__setattr__(self, "_sizes", tuple(int(x) for x in sizes) if all(isinstance(x, Integral) for x in sizes) else None)
         if self.head_map is not None:
             import torch
             m = self.head_map
@@ -89,22 +92,24 @@ class Layout:
 
 # The struct of a layout and its slot size depend on the layout's values alone (the head map
 # enters with the address it has at the call), and the library only reads the struct: both are
-# kept by value.
+# kept by value.  Only for integers (Python's and numpy's): 4.0 would pass for 4 as a key, though it
+# is no size, and a tensor need not keep its value; c() takes those at each call.
 @functools.lru_cache(maxsize=512)
-def _layout_of(H, Hqk, dk, dv, k_hi, fmt, Hm, head_map):
-    return ctypes.pointer(DampLayout(H, Hqk, dk, dv, k_hi, fmt, Hm, head_map))
+def _layout_of(sizes, head_map):
+    return ctypes.pointer(DampLayout(*sizes, head_map))
 
 
 def _cptr(layout):
-    m = layout.head_map
-    return _layout_of(layout.num_heads, layout.num_qk_heads, layout.d_k, layout.d_v, layout.k_hi, layout.lo_format,
-                      layout.model_heads, None if m is None else m.data_ptr())
+    sizes, m = getattr(layout, "_sizes", None), layout.head_map
+    if sizes is None:
+        return ctypes.pointer(layout.c())
+    return _layout_of(sizes, None if m is None else m.data_ptr())
 
 
 @functools.lru_cache(maxsize=512)
-def _slot_bytes_of(H, Hqk, dk, dv, k_hi, fmt, Hm, mapped):
+def _slot_bytes_of(sizes, mapped):
     """Slot size of a pool, 0 for a layout the library does not take (a map's address plays no part)."""
-    return int(lib().damp_slot_bytes(ctypes.pointer(DampLayout(H, Hqk, dk, dv, k_hi, fmt, Hm, 16 if mapped else None))))
+    return int(lib().damp_slot_bytes(ctypes.pointer(DampLayout(*sizes, 16 if mapped else None))))
 
 
 def head_groups(k_hi_of_head, num_qk_heads: int, d_k: int, d_v: int, lo_format: int = LO_U8_AFFINE_G32_H32,
@@ -161,8 +166,7 @@ def _fits_operands(torch, layout, kda, q, k, v, g, beta, o, slot_idx, lead):
 def _fits_pool(torch, layout, state, perm, num_slots, B, slot_idx):
     """state and perm of a packed call, and num_slots (None: all of state's)."""
     n = state.shape[0]
-    sb = _slot_bytes_of(layout.num_heads, layout.num_qk_heads, layout.d_k, layout.d_v, layout.k_hi, layout.lo_format,
-                        layout.model_heads, layout.head_map is not None)
+    sb = _slot_bytes_of(layout._sizes, layout.head_map is not None)
     return (sb > 0 and (num_slots is None or 0 <= num_slots <= n)
             and (slot_idx is not None or B <= (n if num_slots is None else num_slots))
             and _fit(state, (n, sb), torch.uint8) and _fit(perm, (layout.num_heads, layout.d_k), torch.uint8))
