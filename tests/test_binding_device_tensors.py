@@ -67,3 +67,19 @@ def test_a_size_tensor_is_read_at_each_call(calls):
     assert damp._cptr(L).contents.k_hi == K
     k_hi += 2
     assert damp._cptr(L).contents.k_hi == K + 2
+
+
+def test_outputs_are_plain_tensors_whatever_class_v_has(calls):
+    L = _layout()
+    args = dict(stream=_Stream())
+    step, chunk = _dev(_ops("gdn")), _dev(_ops("gdn", (B, T)))
+    heads = _dev(torch.arange(H, dtype=torch.int32))
+    M = damp.Layout(H, HQK, DK, DV, K, model_heads=H, head_map=heads)
+    state, perm = _dev(_pool(L)), _dev(_perm())
+    outs = [damp.gdn_decode_step(L, state, perm, **step, **args), damp.gdn_decode_step(M, state, perm, **step, **args),
+            damp.gdn_decode_step_groups([(M, state, perm)], **step, **args),
+            damp.gdn_prefill_chunk(L, state, perm, **chunk, **args),
+            damp.gdn_prefill_chunk(L, state, perm, lengths=_dev(torch.zeros(B, dtype=torch.int32)), **chunk, **args)]
+    assert len(calls) == len(outs)
+    for o in outs:
+        assert type(o) is torch.Tensor and o.dtype is torch.float32
