@@ -6,7 +6,7 @@ import torch
 
 import paper_2608_27513_gb300 as damp
 from paper_2608_27513_gb300 import _lib, build
-from tests.test_binding_shapes import B, DK, DV, H, HQK, K, T, _NoCompute, _bad_ops, _layout, _ops, _perm, _pool
+from tests.test_binding_shapes import B, DK, DV, H, HQK, K, T, _layout, _NoCompute, _ops, _perm, _pool
 
 
 class _OnGpu(torch.Tensor):
@@ -83,3 +83,94 @@ def test_outputs_are_plain_tensors_whatever_class_v_has(calls):
     assert len(calls) == len(outs)
     for o in outs:
         assert type(o) is torch.Tensor and o.dtype is torch.float32
+
+
+def _fp32_state():
+    return torch.zeros((B, H, DK, DV))
+
+
+def _entries():
+    """(name, call of the keyword arguments, good arguments) of every entry point with quick checks."""
+    L = _layout()
+    heads = _dev(torch.arange(H, dtype=torch.int32))
+    M = damp.Layout(H, HQK, DK, DV, K, model_heads=H, head_map=heads)
+    idx = torch.arange(B, dtype=torch.int32)
+    out = []
+    for kind in ("gdn", "kda"):
+        step, chunk = _ops(kind), _ops(kind, (B, T))
+        fn = lambda name: getattr(damp, name.format(kind))
+        packed = dict(state=_pool(L), perm=_perm(), slot_idx=idx, num_slots=8)
+        out += [
+            (f"{kind} step", lambda state, perm, f=fn("{}_decode_step"), **a: f(L, state, perm, **a),
+             dict(step, o=torch.zeros((B, H, DV)), **packed)),
+            (f"{kind} fp32 step", lambda state, f=fn("fp32_{}_decode_step"), **a: f(L, state, **a),
+             dict(step, state=_fp32_state(), o=torch.zeros((B, H, DV)), slot_idx=idx, num_slots=B)),
+            (f"{kind} chunk", lambda state, perm, f=fn("{}_prefill_chunk"), **a: f(L, state, perm, **a),
+             dict(chunk, o=torch.zeros((B, T, H, DV)), lengths=torch.zeros(B, dtype=torch.int32), **packed)),
+            (f"{kind} group step", lambda state, perm, f=fn("{}_decode_step_groups"), **a: f([(M, state, perm)], **a),
+             dict(step, o=torch.zeros((B, H, DV)), state=_pool(L), perm=_perm(), slot_idx=idx))]
+    out.append(("quantize", lambda S, state, perm, **a: damp.quantize_state(L, S, perm, state, **a),
+                dict(S=_fp32_state(), state=_pool(L), perm=_perm(), slot_idx=idx, num_slots=8)))
+    return out
+
+
+def _wrong(name, t):
+    """The argument with one thing wrong: each dimension one longer and one shorter, a dimension more and
+    one less, another type, not contiguous, not on the GPU."""
+    for d in range(t.dim()):
+        if name == "state" and d == 0:
+            continue  # any number of slots
+        for step in (1, -1):
+            shape = list(t.shape)
+            shape[d] += step
+            yield f"dim {d} {step:+d}", _dev(torch.zeros(shape, dtype=t.dtype))
+    yield "a dimension more", _dev(t[None])
+    yield "a dimension less", _dev(t[0].contiguous())
+    other = {torch.uint8: torch.int8, torch.int32: torch.int64, torch.float32: torch.float64, torch.bfloat16: torch.float16}
+    yield "type", _dev(t.to(other[t.dtype]))
+    if t.dim() > 1:
+        yield "not contiguous", _dev(t.transpose(0, 1).contiguous().transpose(0, 1))
+    yield "on the host", t
+
+
+@pytest.mark.parametrize("i", range(9))
+def test_quick_checks_refuse_one_wrong_argument_at_a_time(calls, monkeypatch, i):
+    """Well-formed arguments pass the quick checks alone (the per-tensor checks are taken out for that
+    call); with any single one wrong the call raises and nothing is launched."""
+    name, call, good = _entries()[i]
+    good = dict(_dev(good), stream=_Stream())
+    with monkeypatch.context() as m:
+        for check in ("_want", "_want_pool", "_want_batch", "_want_operands", "_cuda_contig"):
+            m.setattr(damp, check, lambda *a, **k: pytest.fail(f"{name}: good arguments reached the per-tensor checks"))
+        call(**good)
+        call(**{k: None if k in ("slot_idx", "num_slots", "o", "lengths") else v for k, v in good.items()})
+    assert len(calls) == 2
+    for arg, t in good.items():
+        if not isinstance(t, torch.Tensor):
+            continue
+        for what, bad in _wrong(arg, t.as_subclass(torch.Tensor)):
+            with pytest.raises((ValueError, TypeError)):
+                call(**dict(good, **{arg: bad}))
+            assert len(calls) == 2, (name, arg, what)
+        if arg not in ("slot_idx", "o", "lengths", "perm"):
+            with pytest.raises((ValueError, TypeError, AttributeError)):
+                call(**dict(good, **{arg: None}))
+            assert len(calls) == 2, (name, arg, "missing")
+    slots = good["state"].shape[0]
+    few = dict(good, slot_idx=None, state=_dev(good["state"].as_subclass(torch.Tensor)[:B - 1].clone()))
+    pools = [few] if "num_slots" not in good else [
+        dict(good, num_slots=slots + 1), dict(good, num_slots=-1), dict(good, slot_idx=None, num_slots=B - 1), dict(few, num_slots=None)]
+    for args in pools:
+        with pytest.raises(ValueError):
+            call(**args)
+        assert len(calls) == 2, name
+
+
+def test_operands_of_one_wrong_type_and_groups_without_a_map_are_refused(calls):
+    L = _layout()
+    state, perm, args = _dev(_pool(L)), _dev(_perm()), dict(stream=_Stream())
+    with pytest.raises(TypeError):
+        damp.kda_decode_step(L, state, perm, **_dev(_ops("kda", dt=torch.float16)), **args)
+    with pytest.raises(ValueError, match="head map"):
+        damp.kda_decode_step_groups([(L, state, perm)], **_dev(_ops("kda")), **args)
+    assert calls == []
