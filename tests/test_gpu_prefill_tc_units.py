@@ -1,4 +1,4 @@
-"""The tensor-core prefill's units: the order of a ragged chunk's rows, and what it costs."""
+"""The tensor-core prefill's units: value blocks per unit, the order of a ragged chunk's rows and what it costs."""
 import pytest
 import torch
 
@@ -57,3 +57,37 @@ def test_lengths_cost_little_where_all_rows_are_whole(B):
     lengths = torch.full((B,), T, dtype=torch.int32, device=DEV)
     call = lambda n: (lambda: damp.gdn_prefill_chunk(L, pool, perm, o=o, lengths=n, **ops))
     assert_at_most(call(lengths), call(None), 1.05, f"{B} rows")
+
+
+@pytest.mark.parametrize("kind,what", [("gdn", "plain"), ("gdn", "head map"), ("kda", "plain"), ("kda", "head map"),
+                                       ("kda", "strong decay")])
+@pytest.mark.parametrize("fmt,k_hi", [(0, 40), (1, 16), (3, 10), (4, 0)])
+@pytest.mark.parametrize("B", [8, 40])
+def test_heads_in_two_and_in_four_blocks_equal_heads_in_one(kind, fmt, k_hi, B, what):
+    """A head's value blocks go one, two or four to a unit by the number of (row, head) pairs: 8 pairs
+    (a row of its own: one block, the case that the oracle tests pin), 64 and 320.  Rows of a batch get
+    what they get alone, bit for bit, in every format; for held heads that are a subset of the layer's in
+    another order, and for KDA decays that cut the pieces short."""
+    H, T = 8, 70
+    L, perm, pool, ops, gen = _operands(kind, B, T, H, 80 + B + fmt, fmt, k_hi)
+    if what == "strong decay":
+        ops["g"] *= torch.where(torch.rand(B, 1, H, 1, generator=gen, device=DEV) < 0.5, 60.0, 8.0)
+    rest = slice(0, 0)
+    if what == "head map":
+        Hm = 12
+        L, _, _, ops, _ = _operands(kind, B, T, Hm, 81 + B, fmt, k_hi)
+        held = torch.randperm(Hm, generator=gen, device=DEV)[:H].to(torch.int32)
+        rest = [m for m in range(Hm) if m not in held.tolist()]
+        L = damp.Layout(H, Hm, 128, 128, k_hi, fmt, model_heads=Hm, head_map=held)
+    lengths = torch.randint(1, T + 1, (B,), generator=gen, device=DEV, dtype=torch.int32)
+    lengths[B // 2] = T
+    idx = torch.randperm(B, generator=gen, device=DEV).to(torch.int32)
+    alone = pool.clone()
+    o = _chunk(kind)(L, pool, perm, lengths=lengths, slot_idx=idx, **ops)
+    assert bool(torch.isfinite(o).all())
+    for b in range(B):
+        ob = _chunk(kind)(L, alone, perm, lengths=lengths[b:b + 1].clone(), slot_idx=idx[b:b + 1].clone(),
+                          **{n: t[b:b + 1] for n, t in ops.items()})
+        assert torch.equal(o[b:b + 1], ob), b
+    assert not o[:, :, rest].any()
+    assert torch.equal(pool, alone)
