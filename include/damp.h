@@ -39,8 +39,10 @@
  *   - A kernel never traps.  A slot index outside [0, num_slots) makes the kernel
  *     skip that batch row (its state and outputs are left untouched) and sets
  *     DAMP_DEV_BAD_SLOT in the device status word; a bounded wait inside a kernel
- *     that runs out sets DAMP_DEV_WAIT_TIMEOUT.  damp_device_status() reads and
- *     clears the word.
+ *     that runs out sets DAMP_DEV_WAIT_TIMEOUT, and the rows of o and the states
+ *     that were still to come in that call stay as they were: where the bit is set,
+ *     o is unspecified (an o that was not cleared holds whatever was there before).
+ *     damp_device_status() reads and clears the word.
  *   - Operands are in natural key-channel order; the kernels apply pi.  Inputs
  *     q, k (and v) are read-only; the state is updated in place; o is written.
  *     Batch rows that name the same slot race: slot indices of one call must be

@@ -340,7 +340,8 @@ def _step(fn_name, layout, state, perm, q, k, v, g, beta, o, slot_idx, num_slots
 
 
 def gdn_decode_step(layout, state, perm, q, k, v, g, beta, o=None, slot_idx=None, num_slots=None, stream=None):
-    """One GDN decode step on the packed state (in place); returns o [B, H, d_v] float32."""
+    """One GDN decode step on the packed state (in place); returns o [B, H, d_v] float32, undefined
+    for rows of a slot outside the pool and where device_status() has DEV_WAIT_TIMEOUT set."""
     return _step("damp_gdn_decode_step", layout, state, perm, q, k, v, g, beta, o, slot_idx, num_slots, stream)
 
 
@@ -456,8 +457,10 @@ def _prefill(fn_name, layout, state, perm, q, k, v, g, beta, o, lengths, slot_id
                      ("o", o), ("slot_idx", slot_idx), ("lengths", lengths)):
             _cuda_contig(n, t)
     if o is None:
-        # rows past a length, of a slot outside the pool or of another group's heads stay zero;
-        # without lengths, slot indices and a head map the call writes every row
+        # rows past a length, of a slot outside the pool or of another group's heads stay zero; without
+        # lengths, slot indices and a head map the call writes every row, unless a wait in the kernel
+        # runs out (DEV_WAIT_TIMEOUT): the rows still to come then hold what the allocator left there
+        # (the fill of all rows cost 30 us at 256 x 64 tokens)
         o = _new_output(torch, v, (B, T, layout.heads_of_operands, layout.d_v),
                         lengths is not None or slot_idx is not None or layout.head_map is not None)
     _check(getattr(lib(), fn_name)(_cptr(layout), state.data_ptr(), num_slots, _addr(slot_idx), B, T, _addr(lengths),
@@ -470,7 +473,8 @@ def _prefill(fn_name, layout, state, perm, q, k, v, g, beta, o, lengths, slot_id
 def gdn_prefill_chunk(layout, state, perm, q, k, v, g, beta, o=None, lengths=None, slot_idx=None, num_slots=None,
                       stream=None):
     """One GDN prefill chunk on the packed state (in place): q, k [B, T, H_qk, d_k], v [B, T, H, d_v],
-    g, beta [B, T, H]; returns o [B, T, H, d_v] float32."""
+    g, beta [B, T, H]; returns o [B, T, H, d_v] float32 (rows past a length are zero).  Where
+    device_status() has DEV_WAIT_TIMEOUT set, o is undefined."""
     return _prefill("damp_gdn_prefill_chunk", layout, state, perm, q, k, v, g, beta, o, lengths, slot_idx,
                     num_slots, stream)
 
@@ -578,7 +582,8 @@ def quantize_state(layout, S, perm, state, slot_idx=None, num_slots=None, stream
 
 
 def dequantize_state(layout, state, perm, batch=None, S=None, slot_idx=None, num_slots=None, stream=None):
-    """Reconstruct natural-order FP32 states [B, H, d_k, d_v] from packed slots."""
+    """Reconstruct natural-order FP32 states [B, H, d_k, d_v] from packed slots.  perm must hold a
+    permutation per head: a channel that it leaves out is undefined in an allocated S."""
     import torch
     n_slots = _want_pool(layout, state, num_slots)
     B = (slot_idx.shape[0] if slot_idx is not None else n_slots) if batch is None else int(batch)
@@ -588,8 +593,8 @@ def dequantize_state(layout, state, perm, batch=None, S=None, slot_idx=None, num
     for n, t in (("S", S), ("perm", perm), ("state", state), ("slot_idx", slot_idx)):
         _cuda_contig(n, t)
     if S is None:
-        # rows of a slot outside the pool or of another group's heads stay zero; without slot
-        # indices and a head map the call writes every row
+        # rows of a slot outside the pool or of another group's heads stay zero; without slot indices
+        # and a head map the call writes every row (perm holds permutations, as every call requires)
         alloc = torch.empty if slot_idx is None and layout.head_map is None else torch.zeros
         S = alloc((B, layout.heads_of_operands, layout.d_k, layout.d_v), dtype=torch.float32, device=state.device)
     c = layout.c()
@@ -665,7 +670,8 @@ def unpack_tiers(layout, state, batch=None, slot_idx=None, num_slots=None, strea
 
 
 def device_status() -> int:
-    """Read and clear the device status word (DEV_* bits)."""
+    """Read and clear the device status word (DEV_* bits).  Outputs of the calls since the last
+    reading are undefined where DEV_WAIT_TIMEOUT is set."""
     v = ctypes.c_uint32(0)
     _check(lib().damp_device_status(ctypes.byref(v)), "damp_device_status")
     return int(v.value)
