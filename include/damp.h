@@ -224,11 +224,12 @@ DAMP_API damp_status damp_kda_decode_step(const damp_layout *layout, void *state
  *              (DAMP_ERR_SHAPE otherwise) and lo_format (DAMP_ERR_FORMAT otherwise);
  *              pools must not overlap each other, the operands or o (DAMP_ERR_ALIAS).
  * Two groups with d_k = 128, BF16 operands, lo_format 0 or 1 and K_hi pairs 12/20,
- * 8/24 or 4/28 run as one launch whose CTAs are split between the groups in proportion
- * to their records; other groups run one launch per group.  Results are the same as
- * one damp_gdn_decode_step call per group (the records up to the rounding of a rare
- * float-ordering tie: the one-launch form runs compile-time record layouts), except that in the one-launch form a lost record copy of the first
- * group also leaves the second group's records unwritten (DAMP_DEV_WAIT_TIMEOUT is set).
+ * 8/24 or 4/28 run as one launch in which every warp takes its share of the first group's
+ * records and then its share of the second's; other groups run one launch per group.
+ * Results are the same as one damp_gdn_decode_step call per group (the records up to the
+ * rounding of a rare float-ordering tie: the one-launch form runs compile-time record
+ * layouts), except that in the one-launch form a warp that loses a record copy of the first
+ * group leaves its records of the second unwritten too (DAMP_DEV_WAIT_TIMEOUT is set).
  * Every argument check runs before anything is enqueued.
  */
 DAMP_API damp_status damp_gdn_decode_step_groups(const damp_layout *layouts, int32_t n_groups, void *const *states,

@@ -1,9 +1,9 @@
 // decode_fp32.cu -- the FP32-state step (the deployment baseline of Sec. 6.1: FP32
 // recurrent-state storage) and the FP32 trajectories of a calibration run, GDN and KDA.
 //
-// A unit is up to four value blocks of one (slot, head); a CTA of four warps walks units
-// (persistent), warp w holding a tile of d_k rows x 32 columns in registers over the
-// launch's tokens (one token for a decode step).  Lane (pc, cg) = (lane / 8, lane % 8) holds
+// The pipelined kernel (fp32_tokens_kernel): a unit is up to four value blocks of one (slot,
+// head); a CTA of four warps walks units (persistent), warp w holding a tile of d_k rows x 32
+// columns in registers over the launch's tokens (one token for a decode step).  Lane (pc, cg) = (lane / 8, lane % 8) holds
 // columns 4 cg .. 4 cg + 3 of the rows u = pc mod 4:
 //   * a row is 128 bytes of 16-byte accesses (whole lines in memory, no bank conflicts);
 //   * the sums over the rows run as four chains (rows 0, 4, 8, ..; 1, 5, 9, ..; ...), one
@@ -15,17 +15,17 @@
 // computed from registers and stored; the per-channel operands (k, q, decay, beta k) are
 // staged once per unit and NT tokens from copies made in the same way.
 //
-// Measured (B = 64, H = 32, d = 128, GDN, 268 MB of state per step, more than L2): 46.9 us, 5.8
-// TB/s, bound by HBM; 49.6 us with one column per lane and each tile loaded, computed and
-// stored in turn.  A calibration run over 32 documents (KDA): ~20 us for one token (the 134 MB
-// that the states move through L2), 36 us for eight, 2.6 us per further token -- FP32
-// arithmetic (1.3 us at the FMA rate) and the operand loads, with two warps per scheduler.
-// With one launch per token the eight tokens between two samples took 165 us.
+// Measured (B = 64, H = 32, d = 128, GDN, 268 MB of state per step, more than L2): 45.0 us, 6.0
+// TB/s, bound by HBM; 47.8 us with one column per lane and each tile loaded, computed and
+// stored in turn (fp32_tile_kernel, which stays for shapes that leave these CTAs part empty).  A
+// calibration run over 32 documents (KDA): 16 us for one token (the 134 MB that the states move
+// through L2), 30 us for eight, 2.5 us per further token -- FP32 arithmetic (1.3 us at the FMA
+// rate) and the operand loads, with two warps per scheduler.  With one launch per token eight
+// tokens took 127 us.
 #include "damp_common.cuh"
 #include "damp_internal.h"
 
 #include <algorithm>
-#include <climits>
 
 namespace damp {
 

@@ -10,9 +10,10 @@
 // With L = I + (beta_t f_ts k_t.k_s)_{s<t} (unit lower triangular),
 // M = (f_ts q_t.k_s)_{s<=t} and Y = diag(beta) (V - diag(gamma) K S_0):
 //     U = L^-1 Y,  O = diag(gamma) Q S_0 + M U,  S_C = gamma_C S_0 + K^T diag(f_C.) U.
-// One CTA of eight warps owns a (slot, head) for the whole chunk; its state stays in
-// tensor memory (FP32, lane = record row) from the reconstruction of the packed record
-// to the requantization.  Per piece, four tcgen05.mma products (bf16 operands, FP32
+// One CTA of eight warps owns a unit for the whole chunk: a (slot, head), or one or two of
+// its four value blocks where few heads run (tc_nv).  Its state stays in tensor memory
+// (FP32, lane = record row) from the reconstruction of the packed records to the
+// requantization.  Per piece, four tcgen05.mma products (bf16 operands, FP32
 // accumulation in tensor memory, M = 128):
 //     [K; Q] S_0         -> W = K S_0 (lanes 0-63), P = Q S_0 (lanes 64-127)
 //     [K; Q] K^T         -> K K^T, Q K^T
@@ -22,10 +23,10 @@
 // k and q are bf16 inputs (exact operands); the FP32 operands (S_0, M, U, f_C. U) enter
 // as three bf16 parts x = hi + mid + lo (24 significant bits), and a product of two split
 // operands takes the six partial products down to 2^-16 relative, so the products keep
-// FP32 accuracy.  U = L^-1 Y is solved by forward substitution on the CUDA cores (one
-// thread per value column, in blocks of 16 rows), as are the decay factors
+// FP32 accuracy.  U = L^-1 Y is solved by forward substitution on the CUDA cores (tc_solve:
+// each warp a few rows of all columns, in register tiles), where the decay factors
 // (running products and shuffle scans: no cancellation of cumulative log sums) and the
-// requantization.  With the H_32 formats the whole chunk runs in the transformed domain
+// requantization run too.  With the H_32 formats the whole chunk runs in the transformed domain
 // (S~ = S H, v~ = v H, o = o~ H per value block of 32), as the other prefill kernels do.
 #pragma once
 
@@ -225,8 +226,9 @@ __device__ __forceinline__ uint32_t tc_k64_off(int row, int k) {
 }
 
 // The record rows of a (slot, head) (value-block records at `recs`, `rstride` apart in shared
-// memory) reconstructed into tensor-memory lane u = record row, blocks ca .. cb - 1: FP32 at the natural scale, FP16 rows taken
-// into the H_32 domain with the H_32 formats (where the low tier's codes already are).
+// memory) reconstructed into tensor-memory lane u = record row, blocks ca .. cb - 1: FP32 at the
+// natural scale, FP16 rows taken into the H_32 domain with the H_32 formats (where the low
+// tier's codes already are).
 template <int FMT>
 __device__ __forceinline__ void tc_reconstruct(const PrefillParams &p, uint32_t recs, int rstride, int u, int ca, int cb,
                                                uint32_t tS) {
@@ -474,11 +476,12 @@ __device__ __forceinline__ TcUnit tc_next_unit(const PrefillParams &p, int64_t &
     return n;
 }
 
-// One CTA of kTcThreads threads per (slot, head) unit at a time (persistent over units);
+// One CTA of kTcThreads threads per unit of NV value blocks at a time (persistent over units);
 // d_k = d_v = 128, bf16 q/k/v, low tier FMT (UINT8 or UINT4 affine, with or without H_32;
-// the launchers also instantiate no FP8 or row-absmax kernel).  Thread (row, half):
+// the launchers instantiate no FP8 or row-absmax kernel).  Thread (row, half):
 // row = tensor-memory lane (warps w and w + 4 reach the same lanes), half = 0 / 1 splits
-// a row's value blocks (0-1 / 2-3) or a phase's tasks between the two.
+// a row's value blocks (the unit's first and second half of them; with NV = 1 half 0 has the one) or a
+// phase's tasks between the two.
 template <int FMT, int NV>
 __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_gdn_kernel(const PrefillParams p) {
     static_assert(FMT != kFmtS8Row, "the row-absmax format shares a row scale over the value blocks");

@@ -55,10 +55,12 @@ constexpr int kKdMaxRec = 8192;     // four records fit in [kKdRec, kKdZ)
 constexpr float kKdMaxLog = 85.0f;  // largest log-range of xi on either side of the reference token
 constexpr int kKdThreads = 512;     // four threads per tensor-memory lane (warps w, w + 4, w + 8, w + 12)
 
-// One CTA of kKdThreads threads per (slot, head) unit at a time (persistent over units);
+// One CTA of kKdThreads threads per unit of NV value blocks of a (slot, head) at a time
+// (persistent over units);
 // d_k = d_v = 128, bf16 q/k/v, low tier FMT (UINT8 or UINT4 affine, with or without H_32).
 // Thread (row, quarter qq): row = tensor-memory lane (warps w, w + 4, w + 8 and w + 12
-// reach the same lanes); the quarters split a row's value blocks (one each) or a phase's tasks.
+// reach the same lanes); the quarters split a row's value blocks (one each, quarters past NV none) or
+// a phase's tasks, or take a quarter of the unit's columns each.
 template <int FMT, int NV>
 __global__ void __launch_bounds__(kKdThreads, 1) prefill_tc_kda_kernel(const PrefillParams p) {
     static_assert(FMT != kFmtS8Row, "the row-absmax format shares a row scale over the value blocks");

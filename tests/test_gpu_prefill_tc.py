@@ -76,6 +76,8 @@ def test_kda_strong_decay_shortens_the_pieces(g_scale):
     _run(_kda(f"tck_decay{int(g_scale)}", 1, 2, 2, 12, seed=45), 64, g_scale=g_scale)
 
 
+# (Rows are ordered up to 256 of them, and GDN heads go in one, two or four parts as KDA heads do:
+# test_gpu_prefill_tc_units.py has the edges of both.)
 @pytest.mark.parametrize("kind", ["gdn", "kda"])
 @pytest.mark.parametrize("B,T", [(1, 40), (8, 70), (40, 130), (512, 32), (513, 33)])
 def test_ragged_batches_equal_their_rows_alone(kind, B, T):
