@@ -18,7 +18,7 @@
 // touched 32 different lines.  quantize copies the next tile (cp.async) and dequantize loads the
 // next item's codes while the current one is computed.  B = 64, H = 32, d = 128, K_hi = 16 (134
 // MB FP32 + 41 MB packed): quantize 35.8 us, 4.9 TB/s (B = 256: 128 us, 5.5 TB/s), against 54.8
-// and 169 us with a row per lane from memory; dequantize 38 us against 74 us.  HBM-bound.
+// and 169 us with a row per lane from memory; dequantize 34 us against 73 us.  HBM-bound.
 // pack and unpack, and dequantize at d_k = 32: one warp per record, lane l owns packed rows l, l + 32, ...
 #include "damp_common.cuh"
 #include "damp_internal.h"
@@ -256,12 +256,24 @@ __global__ void __launch_bounds__(32 * kCvWarps) dequantize_kernel(const ConvPar
                                       __float_as_uint(x[2 * m + 1].y)));
             }
             const uint8_t *rec = w.record(k);
+            // FP16 rows, two per 32-bit word: eight words on their way before the first is used (all rows
+            // in FP16: 128 x 128, B = 1 8.8 us, B = 64 38 us; 16.2 and 92 us with one word after the other)
             const int hi_end = min(K, u0 + 32);
-            for (int v = u0; v < hi_end; v += 2) {
-                const float2 f = h2_to_f2(*reinterpret_cast<const uint32_t *>(rec + hi_elem_off(v, lane)));
-                const uint32_t at = tile + (uint32_t)((v - u0) * kCvRow * 4 + 4 * lane);
-                sts32(at, __float_as_uint(f.x));
-                if (v + 1 < K) sts32(at + kCvRow * 4, __float_as_uint(f.y));
+#pragma unroll 1
+            for (int v0 = u0; v0 < hi_end; v0 += 16) {
+                uint32_t hw[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (v0 + 2 * j < hi_end) hw[j] = *reinterpret_cast<const uint32_t *>(rec + hi_elem_off(v0 + 2 * j, lane));
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int v = v0 + 2 * j;
+                    if (v >= hi_end) break;
+                    const float2 f = h2_to_f2(hw[j]);
+                    const uint32_t at = tile + (uint32_t)((v - u0) * kCvRow * 4 + 4 * lane);
+                    sts32(at, __float_as_uint(f.x));
+                    if (v + 1 < K) sts32(at + kCvRow * 4, __float_as_uint(f.y));
+                }
             }
             __syncwarp();
             float *const dst = w.rows(k) + 4 * lc;

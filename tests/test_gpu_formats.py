@@ -10,6 +10,7 @@ import paper_2608_27513_gb300 as damp
 import workloads as wl
 from oracle import core
 from tests import parity as P
+from tests.timing import assert_at_most
 from tests.test_gpu_prefill import _run as run_chunks
 
 pytestmark = pytest.mark.gpu
@@ -167,3 +168,22 @@ def test_dequantize_of_32_channels_matches_oracle(fmt, K):
     want[500] = 0
     scale = np.abs(want).max(axis=-1, keepdims=True) + 1e-30
     assert np.all(np.abs(got - want) <= 1e-6 * scale)
+
+
+@pytest.mark.parametrize("d,batch", [(128, 1), (64, 1), (64, 64)])
+def test_dequantize_of_fp16_rows_keeps_pace_with_codes(d, batch):
+    """All rows in FP16 take at most 1.5 times as long as all rows in codes (half the bytes of the
+    former, which a batch of 64 still reads from L2; above twice where each word is waited for)."""
+    H = 32
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(d)
+    S = torch.randn(batch, H, d, d, generator=gen, device=DEV)
+    perm = torch.stack([torch.randperm(d, generator=gen, device=DEV) for _ in range(H)]).to(torch.uint8)
+
+    def call(K):
+        L = damp.Layout(H, H, d, d, K, 0)
+        pool = damp.new_state(L, batch, DEV)
+        damp.quantize_state(L, S, perm, pool)
+        out = torch.empty_like(S)
+        return lambda: damp.dequantize_state(L, pool, perm, S=out)
+    assert_at_most(call(d), call(0), 1.5, f"{d} x {d}, {batch} slots")
