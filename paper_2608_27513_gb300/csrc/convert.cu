@@ -290,8 +290,10 @@ __global__ void __launch_bounds__(32 * kCvWarps) dequantize_kernel(const ConvPar
 
 // pack and unpack, and dequantize at d_k = 32: a record is a single item there, without a next one
 // for a warp's loads to run ahead to, and the tile only adds its way through shared memory.
+// Packing byte codes at d_k = 32 asks for six CTAs per SM (the compiler's own choice of 48 registers
+// leaves five: 32 x 128, B = 64, H = 32 12.9 us, so 11.9; 32 x 96 7.5 / 6.6).
 template <int R, int FMT, int OP>
-__global__ void __launch_bounds__(256) tiers_kernel(const ConvParams p) {
+__global__ void __launch_bounds__(256, R == 1 && OP == kPackTiers && !fmt_u4(FMT) ? 6 : 0) tiers_kernel(const ConvParams p) {
     constexpr bool HAD = fmt_had(FMT), U4 = fmt_u4(FMT);
     constexpr int CB = U4 ? 16 : 32;  // code bytes per row and value block
     const int lane = threadIdx.x & 31;
