@@ -483,10 +483,24 @@ static cudaError_t launch_fp32_tile(const StepArgs &a, cudaStream_t stream) {
 //   d_k = 32: 32 x 32, B = 256: 40 / 17; 32 x 128: even, from L2 13 / 9.
 // A call of few units gives each its own CTA, where the tile kernel packs eight tiles into one:
 //   128 x 32, B = 8: 5 / 11; 64 x 64, B = 8: 3.6 / 4.3; 128 x 160, B = 2: 9.3 / 11.
+// At d_k = 128 from L2 a wave of CTAs that is part full costs the pipelined kernel as much as a full
+// one, where the tile kernel gives every SM a smaller share (fp32_uneven; 152 SMs, a wave is 304 units):
+//   d_v = 128: 400 units 7.7 / 8.3 us, 432: 9.1 / 8.5, 528: 9.35 / 9.2, 560: 9.4 / 9.5, 784: 12.8 / 12.4,
+//     1024: 14.1 / 15.8;
+//   d_v = 256 (rows copied one by one), GDN: 144 units 9.1 / 10.1, 208: 10.7 / 10.2, 336: 16.9 / 13.7,
+//     496: 18.4 / 16.1, 624: 24.7 / 22.2, 784: 26.0 / 25.7, 816: 26.1 / 27.2; KDA: 304 10.6 / 10.8, 336:
+//     15.9 / 13.8, 528: 17.6 / 17.1, 560: 17.6 / 17.7, 624: 23.2 / 22.3, 720: 23.2 / 24.3.
+static bool fp32_uneven(int64_t V, int64_t units, bool kda) {
+    const int64_t sms = sm_count(), last = units % (2 * sms);
+    if (V == 3) return false;
+    if (V == 4) return units > 2 * sms && units < 6 * sms && 5 * last > 4 * sms && 2 * last <= 3 * sms;
+    return kda ? units > 2 * sms && 5 * units <= 22 * sms && 2 * last <= 3 * sms : units > sms && 4 * units <= 21 * sms;
+}
+
 static bool fp32_pipelined(const StepArgs &a) {
     const int64_t V = a.dv / kG, VG = (V + kFp32Warps - 1) / kFp32Warps, units = (int64_t)a.batch * a.H * VG;
     const bool full = V % kFp32Warps == 0 || V == 3;
-    if (a.dk == 128 && (full || units <= sm_count())) return true;
+    if (a.dk == 128) return units <= sm_count() || (full && !fp32_uneven(V, units, a.kda));
     if (a.dk < 64 || VG > 1) return false;
     return units <= 2 * sm_count() || (full && (int64_t)a.batch * a.H * a.dk * a.dv * 4 > kFp32L2Bytes);
 }

@@ -33,7 +33,9 @@ def _workload(kind, dk, dv, batch, dtype="bf16", heads=32, qk_heads=16):
     ("gdn", 128, 128, "bf16", 40), ("kda", 128, 128, "fp32", 40), ("gdn", 128, 96, "bf16", 40),
     ("kda", 128, 256, "bf16", 40), ("kda", 64, 128, "bf16", 130), ("gdn", 64, 96, "fp32", 170),
     ("gdn", 128, 160, "bf16", 40), ("kda", 128, 64, "bf16", 40), ("gdn", 64, 64, "bf16", 40),
-    ("kda", 32, 32, "fp32", 80), ("gdn", 32, 288, "bf16", 40)])
+    ("kda", 32, 32, "fp32", 80), ("gdn", 32, 288, "bf16", 40),
+    # a part-full wave of the pipelined kernel's CTAs: a warp per tile, rows alone pipelined
+    ("gdn", 128, 128, "bf16", 14), ("kda", 128, 256, "bf16", 8), ("gdn", 128, 384, "fp32", 7)])
 def test_rows_of_a_large_step_equal_their_own_call(kind, dk, dv, dtype, batch):
     """Every row of a large step over scattered slots gets what a call of its own gives it, bit for
     bit, and three rows what the oracle gives them; rows whose slot is outside the pool are left
@@ -89,6 +91,22 @@ def test_narrow_states_keep_pace_with_square_ones(dk, dv, batch, square_batch):
         return lambda: damp.fp32_gdn_decode_step(L, S, d["q"], d["k"], d["v"], d["g"], d["beta"], o=o)
     assert batch * dk * dv == square_batch * 128 * 128
     assert_at_most(call(dk, dv, batch), call(128, 128, square_batch), 2.0, f"{dk} x {dv}")
+
+
+@pytest.mark.parametrize("kind", ["gdn", "kda"])
+def test_a_part_full_wave_costs_little(kind):
+    """320 units of 128 x 256 states (two CTAs per SM and a few units more) take at most 2.05 times
+    as long as 128 x 128 states of the same bytes: 1.85 with a warp per tile, 2.2 where the last few
+    units cost the pipelined kernel as much as a whole wave."""
+    def call(v, b):
+        w = _workload(kind, 128, v, b, heads=16, qk_heads=16)
+        L = damp.Layout(16, 16, 128, v, 0, 0)
+        d = wl.torch_step_inputs(w, 1, DEV)[0]
+        S = torch.zeros(b, 16, 128, v, device=DEV)
+        o = torch.empty(b, 16, v, device=DEV)
+        step = damp.fp32_kda_decode_step if kind == "kda" else damp.fp32_gdn_decode_step
+        return lambda: step(L, S, d["q"], d["k"], d["v"], d["g"], d["beta"], o=o)
+    assert_at_most(call(256, 10), call(128, 20), 2.05, kind)
 
 
 @pytest.mark.parametrize("kind,dk,dv,T,every", [("kda", 128, 128, 21, 8), ("gdn", 128, 160, 17, 8), ("gdn", 64, 96, 7, 2),
