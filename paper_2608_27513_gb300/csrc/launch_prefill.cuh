@@ -36,7 +36,16 @@ static cudaError_t launch_prefill_cg(const PrefillParams &p0, const StepArgs &a,
     int warps = kPrefillWarps;
     while (warps > 1 && warps * warp_smem > max_smem_per_block()) --warps;
     if (warps * warp_smem > max_smem_per_block()) return cudaErrorInvalidValue;
-    const int grid = (int)std::min<int64_t>(p.total_tiles, (int64_t)sm_count());
+    // Up to four tiles per SM: as many warps in a CTA as an SM has tiles, so that each is on a scheduler
+    // of its own (eight warps put the tiles on every second or fourth one: two then share a scheduler;
+    // KDA 128 x 64, 5 rows of 32 heads, 200 tokens: 233 us, so 160).  Above that KDA at d_k = 128 is
+    // faster with full CTAs on fewer SMs (10 rows: 229 us on all SMs, so 217), the others are not (GDN
+    // 198 / 201, 64 x 64 KDA 136 / 139).
+    const int64_t per_sm = (p.total_tiles + sm_count() - 1) / sm_count();
+    int64_t want = p.total_tiles;
+    if (per_sm <= 4) warps = std::min(warps, (int)per_sm);
+    else if (KDA && a.dk == 128) want = (p.total_tiles + warps - 1) / warps;
+    const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count());
     const int smem = warp_smem * warps;
     void (*kern)(PrefillParams) = nullptr;
     if (a.dk == 64) kern = a.in_bf16 ? prefill_cg_kernel<64, KDA, HAD, true> : prefill_cg_kernel<64, KDA, HAD, false>;

@@ -9,6 +9,7 @@ import paper_2608_27513_gb300 as damp
 import workloads as wl
 from oracle import runs
 from tests import parity as P
+from tests.timing import assert_at_most
 
 pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda:0")
@@ -130,3 +131,50 @@ def test_decode_after_prefill_reads_the_chunk_state():
     P.compare_tiers(w, new_ref, P.tiers_from_dev(w, damp.unpack_tiers(L, state), w.batch * w.heads), lo_pre, stats,
                     "decode after prefill")
     stats.check_fraction()
+
+
+def _long_chunk(kind, dk, dv, B, H, T):
+    """Layout, pi, pool and operands of a chunk that the channel-ordered per-token kernel runs."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(dk + dv + B)
+    n = lambda *s: torch.randn(*s, generator=gen, device=DEV)
+    unit = lambda x: (x / x.norm(dim=-1, keepdim=True)).bfloat16()
+    ops = dict(q=unit(n(B, T, H, dk)), k=unit(n(B, T, H, dk)), v=n(B, T, H, dv).bfloat16(),
+               g=-torch.nn.functional.softplus(n(B, T, H) if kind == "gdn" else n(B, T, H, dk) - 3.0),
+               beta=torch.sigmoid(n(B, T, H)))
+    L = damp.Layout(H, H, dk, dv, 10, 0)
+    perm = torch.stack([torch.randperm(dk, generator=gen, device=DEV) for _ in range(H)]).to(torch.uint8)
+    pool = damp.new_state(L, B, DEV)
+    damp.quantize_state(L, 0.1 * n(B, H, dk, dv), perm, pool)
+    return L, perm, pool, ops, gen
+
+
+# 152 SMs: one tile per SM and less, two and three, four, more (KDA, d_k = 128: full CTAs), above eight
+@pytest.mark.parametrize("kind,dk,dv,B,H", [("gdn", 64, 64, 9, 8), ("kda", 128, 96, 16, 8), ("gdn", 128, 32, 57, 8),
+                                            ("kda", 64, 32, 76, 8), ("kda", 128, 64, 47, 8), ("gdn", 64, 96, 40, 8),
+                                            ("kda", 128, 32, 153, 8)])
+def test_rows_of_a_long_chunk_equal_their_own_call(kind, dk, dv, B, H):
+    """Warps per CTA and CTAs follow the number of tiles: every row of a ragged chunk gets what a call of
+    its own (a tile per CTA) gives it, bit for bit."""
+    T = 35
+    L, perm, pool, ops, gen = _long_chunk(kind, dk, dv, B, H, T)
+    fn = damp.kda_prefill_chunk if kind == "kda" else damp.gdn_prefill_chunk
+    lengths = torch.randint(0, T + 1, (B,), generator=gen, device=DEV, dtype=torch.int32)
+    lengths[0] = T
+    alone = pool.clone()
+    o = fn(L, pool, perm, lengths=lengths, **ops)
+    for b in range(B):
+        ob = fn(L, alone[b:b + 1], perm, lengths=lengths[b:b + 1].clone(), **{n: t[b:b + 1] for n, t in ops.items()})
+        assert torch.equal(o[b:b + 1], ob), b
+    assert torch.equal(pool, alone)
+
+
+@pytest.mark.parametrize("B,other,factor", [(5, 2, 1.2), (10, 16, 1.03)])
+def test_tiles_of_a_long_chunk_do_not_share_schedulers_early(B, other, factor):
+    """KDA 128 x 64, 200 tokens: two tiles per SM take as long as one (1.5 times where both are on one
+    scheduler), and four to five no longer than seven (1.06 times where they are spread over all SMs)."""
+    def call(rows):
+        L, perm, pool, ops, _ = _long_chunk("kda", 128, 64, rows, 32, 200)
+        o = torch.empty(rows, 200, 32, 64, device=DEV)
+        return lambda: damp.kda_prefill_chunk(L, pool, perm, o=o, **ops)
+    assert_at_most(call(B), call(other), factor, f"{B} rows")
