@@ -310,9 +310,11 @@ cudaError_t launch_calib_error_energy(const float *S, int32_t batch, int32_t H, 
 cudaError_t launch_calib_log_decay(const float *g, int32_t batch, int32_t H, int32_t Hm, const int32_t *head_map,
                                    int32_t dk, int32_t kda, float *G_acc, cudaStream_t stream) {
     // The ring's start and, for GDN, a warp's 32 rows of G_acc cost more than few rows take, ring /
-    // thread per accumulator: KDA 1 row 2.3 / 1.9 us, 12 rows 2.4 / 2.4, 64 rows 2.6 / 4.5; GDN 1 row
-    // 10.4 / 1.8, 256 rows 12.6 / 5.2, 1500 rows 24.0 / 22.9, 2048 rows 28.6 / 30.1 (32 heads, d_k 128).
-    if (batch < (kda ? 12 : 1792)) {
+    // thread per accumulator: KDA 1 row 2.3 / 1.9 us, 12 rows 2.2 / 2.1, 13 and 15 rows 2.3 / 2.3 and
+    // 2.4, 40 rows 2.6 / 3.2; GDN 1 row 10.4 / 1.8, 256 rows 12.6 / 5.2, 1500 rows 24.0 / 22.9, 2048 rows
+    // 28.6 / 30.1 (32 heads, d_k 128).  At d_k = 64 with a full warp of heads the rows of G_acc take
+    // longer: 1800 rows 30.0 / 26.4, 2200 33.6 / 31.8, 2600 37.1 / 37.2 (24 heads: 27.1 / 26.6 at 1800).
+    if (batch < (kda ? 13 : dk == 64 && H > 24 ? 2560 : 1792)) {
         const int64_t n = (int64_t)H * dk;
         calib_log_decay_few_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(g, batch, H, Hm, head_map, dk, kda,
                                                                                       G_acc);

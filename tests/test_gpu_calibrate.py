@@ -178,7 +178,8 @@ def test_log_decay_sums_in_row_order(rows, kda):
     assert np.array_equal(G, ref if kda else np.repeat(ref[:, None], dk, axis=1))
 
 
-@pytest.mark.parametrize("kda,rows", [(True, 11), (True, 12), (True, 13), (False, 1791), (False, 1792), (False, 1800),
+@pytest.mark.parametrize("kda,rows", [(True, 11), (True, 12), (True, 13), (False, 2559), (False, 2560),
+                                      (False, 1791), (False, 1792), (False, 1800),
                                       (False, 2111)])
 def test_log_decay_sums_on_both_sides_of_the_line(kda, rows):
     """Few rows (a thread per accumulator) and many (the ring) add in the same order."""
@@ -200,3 +201,13 @@ def test_few_rows_of_scalar_gates_take_no_longer_than_of_channel_gates(rows):
     G = torch.zeros((H, dk), device=DEV)
     gdn, kda = -torch.rand(rows, H, device=DEV), -torch.rand(rows, H, dk, device=DEV)
     assert_at_most(lambda: damp.calib_log_decay(L, gdn, G), lambda: damp.calib_log_decay(L, kda, G), 2.0, f"{rows} rows")
+
+
+def test_log_decay_sums_grow_with_the_rows():
+    """Twenty rows above 1780 add at most 5 % to the sums of 32 heads' scalar gates, 64 channels (14 %
+    where the ring of row copies takes over too early)."""
+    H, dk = 32, 64
+    L = damp.Layout(H, H, dk, 64, 0, 0)
+    G = torch.zeros((H, dk), device=DEV)
+    few, more = -torch.rand(1780, H, device=DEV), -torch.rand(1800, H, device=DEV)
+    assert_at_most(lambda: damp.calib_log_decay(L, more, G), lambda: damp.calib_log_decay(L, few, G), 1.05, "1800 rows")
