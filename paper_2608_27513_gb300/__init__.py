@@ -71,14 +71,18 @@ class Layout:
     head_map: object = field(default=None, compare=False, repr=False)
 
     def __post_init__(self):
-        sizes = (self.num_heads, self.num_qk_heads, self.d_k, self.d_v, self.k_hi, self.lo_format, self.model_heads)
-        object.__setattr__(self, "_sizes", tuple(int(x) for x in sizes) if all(isinstance(x, Integral) for x in sizes) else None)
         if self.head_map is not None:
             import torch
             m = self.head_map
             if (not isinstance(m, torch.Tensor) or m.dtype != torch.int32 or not m.is_cuda or not m.is_contiguous()
                     or m.shape != (self.num_heads,)):
                 raise ValueError(f"head_map must be a contiguous int32 CUDA tensor of shape [{self.num_heads}]")
+
+    @functools.cached_property
+    def _sizes(self):
+        """The struct's integers (a call looks them up once per layout), None where one is no integer."""
+        sizes = (self.num_heads, self.num_qk_heads, self.d_k, self.d_v, self.k_hi, self.lo_format, self.model_heads)
+        return tuple(int(x) for x in sizes) if all(isinstance(x, Integral) for x in sizes) else None
 
     @property
     def heads_of_operands(self) -> int:

@@ -69,6 +69,15 @@ def test_a_size_tensor_is_read_at_each_call(calls):
     assert damp._cptr(L).contents.k_hi == K + 2
 
 
+def test_a_layout_looks_up_its_sizes_at_its_first_call(calls):
+    """Making a layout does no more than store its fields; equal layouts stay equal afterwards."""
+    L = _layout()
+    assert "_sizes" not in vars(L)
+    damp.kda_decode_step(L, _dev(_pool(L)), _dev(_perm()), **dict(_dev(_ops("kda")), stream=_Stream()))
+    assert "_sizes" in vars(L)
+    assert L == _layout() and hash(L) == hash(_layout())
+
+
 def test_outputs_are_plain_tensors_whatever_class_v_has(calls):
     L = _layout()
     args = dict(stream=_Stream())
