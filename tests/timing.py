@@ -7,6 +7,7 @@ def best_us(fn, calls=20, reps=5):
     """Smallest time of one fn() in us, from a CUDA graph of `calls` of them."""
     stream = torch.cuda.Stream()
     graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()  # the inputs were made on another stream
     with torch.cuda.stream(stream):
         fn()
         torch.cuda.synchronize()
