@@ -63,7 +63,7 @@ constexpr int kTcRowY = 132;    // floats per row of Y / U
 constexpr int kTcRowV = 272;    // bytes per row of v
 constexpr int kTcMaxSort = 256;  // batch rows up to which a ragged chunk's units are ordered by length
 constexpr int kSmOrder = kSmScal + 1472;
-constexpr int kTcSmem = kSmOrder + 2 * kTcMaxSort;
+constexpr int kTcSmem = kSmOrder + 2 * kTcMaxSort + 16;
 constexpr int kTcMaxRec = 8192; // largest record (d_k = 128): four fit in [kSmRec, kSmV)
 __host__ __device__ constexpr int tc_rec_stride(int rec_bytes) { return (rec_bytes + 127) & ~127; }
 
@@ -413,14 +413,25 @@ __device__ __forceinline__ void tc_requantize(const PrefillParams &p, uint8_t *g
 // head by head through the batch rows, and for a ragged chunk through the rows by falling length
 // (up to kTcMaxSort rows: `order`, uint16 in shared memory, filled by tc_sort_rows), so that the
 // CTAs with the longest units get the shortest ones next.  KDA, 13 rows of up to 133 tokens x 32
-// heads (416 units on 152 SMs): 176 us in batch order, 134 us so.
+// heads (416 units on 152 SMs): 176 us in batch order, 134 us so.  A last round after two, four, .. of
+// them that has not a unit for every CTA starts at the end whose CTAs have fewer 64-token pieces so
+// far (10 rows x 32 heads, one row of 65 tokens, the others within a piece: KDA 94 us where the CTAs
+// with the longest units take those as well, 72 so).  Units that all run at once keep batch order.
 // The order's cost grows with the square of the rows, in every CTA: 1.7 us for 256 rows (from shared
 // memory, one comparison per pair; 3.4 us before), 15 us for 512 from global memory (GDN, 512 rows of
 // 64 tokens x 2 heads: 114.5 us in batch order, 129 us so), where each CTA has enough units that
 // their order matters little.
+// After the rows: 1 if that last round starts at the other end, else 0.
 __device__ __forceinline__ void tc_sort_rows(const PrefillParams &p, uint32_t order, uint32_t scratch) {
     // (length, up to 2^22; the earlier of equal rows) as one number, larger first and distinct
     static_assert(kTcMaxSort <= 512, "a row's number takes nine bits of its key");
+    const int units = p.batch * p.H, grid = (int)gridDim.x, full = units / grid;  // (fits: at most kTcMaxSort rows)
+    if (units <= grid) {  // (also wherever NV < 4)
+        for (int b = threadIdx.x; b < p.batch; b += blockDim.x)
+            asm volatile("st.shared.u16 [%0], %1;" ::"r"(order + 2 * b), "h"((unsigned short)b) : "memory");
+        if (threadIdx.x == 0) asm volatile("st.shared.u16 [%0], %1;" ::"r"(order + 2 * kTcMaxSort), "h"((unsigned short)0) : "memory");
+        return;
+    }
     const int n4 = (p.batch + 3) & ~3;
     for (int b = threadIdx.x; b < n4; b += blockDim.x)  // keys past the batch: 0, below every row's
         sts32(scratch + 4 * b, b < p.batch ? (uint32_t)min(min(max(p.lengths[b], 0), p.T), (1 << 22) - 1) * 512u + 512u - (uint32_t)b : 0u);
@@ -434,6 +445,21 @@ __device__ __forceinline__ void tc_sort_rows(const PrefillParams &p, uint32_t or
             rank += (w.x > key) + (w.y > key) + (w.z > key) + (w.w > key);
         }
         asm volatile("st.shared.u16 [%0], %1;" ::"r"(order + 2 * rank), "h"((unsigned short)b) : "memory");
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int first = 0, last = 0;  // pieces of the first and the last CTA in the full rounds
+        if (full >= 2 && full <= 8 && !(full & 1)) {
+            for (int i = 0; i < full; ++i) {
+                auto pieces = [&](int blk) {
+                    const uint32_t row = lds_u16(order + 2u * (uint32_t)((i * grid + blk) / p.H));
+                    return (int)(((lds32(scratch + 4 * row) - 1u) / 512u + kTcC - 1) / kTcC);
+                };
+                first += pieces((i & 1) ? grid - 1 : 0);
+                last += pieces((i & 1) ? 0 : grid - 1);
+            }
+        }
+        asm volatile("st.shared.u16 [%0], %1;" ::"r"(order + 2 * kTcMaxSort), "h"((unsigned short)(first > last)) : "memory");
     }
 }
 struct TcUnit {
@@ -458,7 +484,8 @@ __device__ __forceinline__ TcUnit tc_next_unit(const PrefillParams &p, int64_t &
     const int HS = p.H * S;
     const int64_t units = (int64_t)p.batch * HS, grid = gridDim.x;
     for (; round * grid < units && !n.ok; ++round) {
-        const int64_t at = round * grid + ((round & 1) ? grid - 1 - blockIdx.x : blockIdx.x);
+        const bool turned = (round & 1) || (sorted && (round + 1) * grid > units && lds_u16(order + 2 * kTcMaxSort));
+        const int64_t at = round * grid + (turned ? grid - 1 - blockIdx.x : blockIdx.x);
         if (at >= units) continue;
         const int r = (int)(at / HS), hs = (int)(at - (int64_t)r * HS);
         n.h = hs / S;

@@ -50,7 +50,7 @@ constexpr int kKdYU = 0;            // Y, then U: 64 rows of kTcRowY FP32
 __host__ __device__ constexpr int kd_bu(int part) { return part == 2 ? 135168 : 16384 * part; }  // U: three bf16 parts, K-major (value columns x tokens)
 constexpr int kKdScal = 208896;     // beta, pi, gamma_m, xi_C, mbarriers, TMEM address
 constexpr int kKdOrder = kKdScal + 2048;
-constexpr int kKdSmem = kKdOrder + 2 * kTcMaxSort;
+constexpr int kKdSmem = kKdOrder + 2 * kTcMaxSort + 16;
 constexpr int kKdMaxRec = 8192;     // four records fit in [kKdRec, kKdZ)
 constexpr float kKdMaxLog = 85.0f;  // largest log-range of xi on either side of the reference token
 constexpr int kKdThreads = 512;     // four threads per tensor-memory lane (warps w, w + 4, w + 8, w + 12)

@@ -59,6 +59,20 @@ def test_lengths_cost_little_where_all_rows_are_whole(B):
     assert_at_most(call(lengths), call(None), 1.05, f"{B} rows")
 
 
+@pytest.mark.parametrize("kind", ["gdn", "kda"])
+def test_one_longer_row_shares_no_cta_of_the_last_round(kind):
+    """Ten rows of 32 heads are two units for every CTA and a third for a few.  One row with a token in a
+    second piece costs at most 12 % (20 % and more where the CTAs with its units get the third ones)."""
+    B, H, T = 10, 32, 65
+    L, perm, pool, ops, _ = _operands(kind, B, T, H, 9)
+    o = torch.empty(B, T, H, 128, device=DEV)
+    even = torch.full((B,), 60, dtype=torch.int32, device=DEV)
+    one = even.clone()
+    one[5] = T
+    call = lambda n: (lambda: _chunk(kind)(L, pool, perm, o=o, lengths=n, **ops))
+    assert_at_most(call(one), call(even), 1.12, kind)
+
+
 @pytest.mark.parametrize("kind,what", [("gdn", "plain"), ("gdn", "head map"), ("kda", "plain"), ("kda", "head map"),
                                        ("kda", "strong decay")])
 @pytest.mark.parametrize("fmt,k_hi", [(0, 40), (1, 16), (3, 10), (4, 0)])
