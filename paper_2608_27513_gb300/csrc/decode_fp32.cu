@@ -19,9 +19,9 @@
 // TB/s, bound by HBM; 47.8 us with one column per lane and each tile loaded, computed and
 // stored in turn (fp32_tile_kernel, which stays for shapes that leave these CTAs part empty).  A
 // calibration run over 32 documents (KDA): 16 us for one token (the 134 MB that the states move
-// through L2), 30 us for eight, 2.5 us per further token -- FP32 arithmetic (1.3 us at the FMA
-// rate) and the operand loads, with two warps per scheduler.  With one launch per token eight
-// tokens took 127 us.
+// through L2) and 2.1 us for each further one up to eight (31 us), 2.5 us in longer runs, whose
+// operands come eight tokens at a time -- FP32 arithmetic (1.3 us at the FMA rate) and the operand
+// loads, with two warps per scheduler.  With one launch per token eight tokens took 127 us.
 #include "damp_common.cuh"
 #include "damp_internal.h"
 
