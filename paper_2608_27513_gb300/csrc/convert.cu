@@ -290,10 +290,8 @@ __global__ void __launch_bounds__(32 * kCvWarps) dequantize_kernel(const ConvPar
 
 // pack and unpack, and dequantize at d_k = 32: a record is a single item there, without a next one
 // for a warp's loads to run ahead to, and the tile only adds its way through shared memory.
-// Packing byte codes at d_k = 32 asks for six CTAs per SM (the compiler's own choice of 48 registers
-// leaves five: 32 x 128, B = 64, H = 32 12.9 us, so 11.9; 32 x 96 7.5 / 6.6).
 template <int R, int FMT, int OP>
-__global__ void __launch_bounds__(256, R == 1 && OP == kPackTiers && !fmt_u4(FMT) ? 6 : 0) tiers_kernel(const ConvParams p) {
+__global__ void __launch_bounds__(256) tiers_kernel(const ConvParams p) {
     constexpr bool HAD = fmt_had(FMT), U4 = fmt_u4(FMT);
     constexpr int CB = U4 ? 16 : 32;  // code bytes per row and value block
     const int lane = threadIdx.x & 31;
@@ -312,8 +310,11 @@ __global__ void __launch_bounds__(256, R == 1 && OP == kPackTiers && !fmt_u4(FMT
             bad_slot = true;
             continue;
         }
-        const int mh = OP == kDequantize && p.head_map ? p.head_map[h] : h;  // row of S
-        if (OP == kDequantize && (mh < 0 || mh >= p.Hm)) {
+        // row of S; pack and unpack have no map and always pass, but without the check the compiler orders
+        // their accesses worse (pack, H = 32: 128 x 96, B = 64 20.9 us, so 19.1; 128 x 64, B = 100 23.2 / 21.0)
+        // and takes 48 registers for 40 at d_k = 32 (32 x 96, B = 64 7.5 / 6.6)
+        const int mh = p.head_map ? p.head_map[h] : h;
+        if (mh < 0 || mh >= p.Hm) {
             bad_head = true;
             continue;
         }
@@ -323,6 +324,7 @@ __global__ void __launch_bounds__(256, R == 1 && OP == kPackTiers && !fmt_u4(FMT
             const int u = lane + 32 * i;
             if (u < K) continue;  // FP16 rows: column-mapped loop below
             const int r = u - K;
+            uint8_t *crec = rec + p.codes_off + lo_chunk_off(r, 0, lo), *crec1 = rec + p.codes_off + lo_chunk_off(r, 1, lo);
             uint32_t *mrec = reinterpret_cast<uint32_t *>(rec + p.meta_off + 4 * r);
             if (OP == kDequantize) {
                 const int n = p.perm[(int64_t)h * p.dk + u] & (p.dk - 1);  // d_k is a power of two
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(256, R == 1 && OP == kPackTiers && !fmt_u4(FMT
                 uint32_t *mrow = reinterpret_cast<uint32_t *>(p.meta) + (((int64_t)b * p.H + h) * lo + r) * p.V + c;
 #pragma unroll
                 for (int m = 0; m < CB / 16; ++m) {
-                    uint32_t *r4 = reinterpret_cast<uint32_t *>(rec + p.codes_off + lo_chunk_off(r, m, lo));
+                    uint32_t *r4 = reinterpret_cast<uint32_t *>(m ? crec1 : crec);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         if (OP == kPackTiers) r4[e] = crow[4 * m + e];
